@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/gbfft.h"
+#include "mixr_plan.h"
 #include "tile_fft.cuh"
 
 namespace gbfft {
@@ -41,7 +42,8 @@ enum PlanKind {
   KIND_MIXED_PASSES = 6   // strided mixed-radix passes: four-step 1-D or 2-D (mixed4.cu)
 };
 
-// Lengths N = 2^a 3^b 5^c 7^d that are not powers of two (mixed.cu).
+// One-pass lengths N = 2^a 3^b 5^c 7^d (mixed.cu): FP64, and the FP32
+// lengths of mixed_ct.cu.
 constexpr int kMixedMaxPasses = 16;
 constexpr long long kMixedMaxN = 14336;   // two shared-memory buffers of N complex values fit
 constexpr long long kMixedMaxN64 = 7168;  // the same for FP64 (complex128) values
@@ -62,6 +64,52 @@ struct MixedArgs {
   double sx, sy;      // output scale (1/N of Eq. 2 exact to FP64 for the FP64 kernel)
   float fsx, fsy;     // the same rounded to FP32 for the FP32 kernel
 };
+// One launch of the FP32 mixed-radix tile kernel (mixr.cuh).
+struct MixrArgs {
+  const float2* in;
+  float2* out;
+  const float2* tw;            // twiddle bases of every pass, pass s at tw_off[s]
+  int N, C;                    // length; columns per CTA
+  int csh, pitch, in_rows;     // strided tiles: C == 2^csh, tile row pitch, input columns are contiguous rows
+  int nrad;
+  int rad[mixr::kMaxPasses];
+  unsigned nb[mixr::kMaxPasses], nb_m[mixr::kMaxPasses];   // N/R and its reciprocal (fdiv)
+  unsigned ns[mixr::kMaxPasses], ns_m[mixr::kMaxPasses];   // Ns and its reciprocal
+  unsigned tw_off[mixr::kMaxPasses];
+  long long ncols;             // columns (strided: per batch)
+  long long tile0;             // first tile of the launch
+  // strided tiles: element (column c, row n) of batch b at b*bs + c*cs + n*ns
+  long long tiles_per_batch, in_bs, out_bs;
+  unsigned in_cs, in_ns, out_cs, out_ns;
+  // four-step twiddle W_Nt^{col k} of output k: dense table ft[k * ft_cols + col], or two
+  // levels ft_lo[e & (2^ft_s - 1)] * ft_hi[e >> ft_s], e = col k < Nt < 2^32, or none
+  const float2* ft;
+  unsigned ft_cols;
+  const float2* ft_lo;
+  const float2* ft_hi;
+  int ft_s;
+  int conj_in, scale_out;
+  float sx, sy;
+};
+struct MixrLaunch {
+  MixrArgs a;
+  const void* fn;
+  int threads, smem;
+  long long ntiles;
+};
+// Strided layout of a pass: batches of ncols columns.
+struct MixrLayout {
+  long long in_bs, in_cs, in_ns, out_bs, out_cs, out_ns;
+};
+size_t mixr_table_entries(const MixrArgs& a);
+int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, const MixrLayout* lay);
+float mixr_strided_cost(long long N, long long ncols, long long batches, bool in_rows);
+int mixr_fill_tables(MixrLaunch& L, float2* tab, cudaStream_t s);
+int mixr_launch(const MixrLaunch& L, const float2* in, float2* out, int conj, float sx, float sy, int scale_out,
+                cudaStream_t s);
+cudaError_t launch_gen_mixr_twiddles(float2* tab, int R, int Ns, cudaStream_t s);
+cudaError_t launch_gen_four_step(float2* tab, long long N, int n1, int n2, cudaStream_t s);
+
 // Mixed-radix lengths with a compile-time three-pass schedule (mixed_ct.cu).
 struct MixedCtInfo {
   long long N;
@@ -102,16 +150,8 @@ struct Mixed4Pass {
   int in_role, out_role;       // 0 the caller's input, 1 its output, 2 the workspace
 };
 constexpr int kMixed4MaxPasses = 2;
-// FP32 sub-lengths with a compile-time schedule (mixed4_ct.cu)
-struct Mixed4CtInfo {
-  long long L;
-  int r0, r1, r2;  // radices (r2 == 1: two passes)
-  int csh;         // 2^csh columns per CTA
-  const void* fn;  // kernel void(Mixed4Args)
-};
-const Mixed4CtInfo* mixed4_ct_lookup(long long L);
-// kernel for element type (FP64 or FP32), 2^csh columns per CTA, padded index
-const void* mixed4_kernel_fn(bool fp64, int csh, bool pad);
+// FP64 kernel, 2^csh columns per CTA, padded index
+const void* mixed4_kernel_fn64(int csh, bool pad);
 int mixed4_plan_1d(fft_plan* p);
 int mixed4_plan_2d(fft_plan* p);
 int mixed4_exec(fft_plan* p, const void* in, void* out, int conj, double sx, double sy, int scale_out,
@@ -192,6 +232,7 @@ struct fft_plan {
   gbfft::MixedArgs mixed;
   int mixed_threads, mixed_smem, mixed_pad;
   const gbfft::MixedCtInfo* mixed_ct;   // compile-time schedule for this length (FP32), or NULL
+  gbfft::MixrLaunch mr[2];   // FP32 mixed radix: one tile pass, or the two passes of a split
   gbfft::Mixed4Pass m4[gbfft::kMixed4MaxPasses];   // KIND_MIXED_PASSES
   int m4n;
   long long m4_n1, m4_n2;   // four-step: column length N1, row length N2 (N = N1 N2); 2-D: ny, nx

@@ -1,10 +1,10 @@
-// mixed.cu -- transforms whose length is not a power of two but a product
-// N = 2^a 3^b 5^c 7^d (N <= 14336), one on-chip pass per transform; the same
-// kernel in FP64 (complex128) for every such N <= 7168, powers of two
-// included.
+// mixed.cu -- transforms of one on-chip pass whose length is a product
+// N = 2^a 3^b 5^c 7^d: plans of FP32 lengths that are not powers of two
+// (N <= 14336; kernels in mixr.cuh and mixed_ct.cu), and the FP64 (complex128)
+// kernel for every such N <= 7168, powers of two included.
 //
 // Eq. 1 holds for any N; the paper's Cooley-Tukey split (Sec. 2.1) works for
-// any factorisation N = R_1 R_2 ... R_s.  These kernels run the same Stockham
+// any factorisation N = R_1 R_2 ... R_s.  The FP64 kernel runs the same Stockham
 // autosort recurrence as the power-of-two tiles (natural order in and out),
 // with the radix of every pass chosen at run time from {16, 8, 4, 2, 3, 5, 7}:
 //   pass with radix R, Ns = product of the earlier radices, butterfly j:
@@ -13,14 +13,11 @@
 //     b[(j div Ns) Ns R + (j mod Ns) + q Ns] = V[q].
 // The first pass reads global memory, the last writes it; the passes in
 // between go through two shared-memory buffers in turn.  Twiddles come from
-// one table W_N^m, m < N (FP64 sincospi rounded once to FP32), since
+// one table W_N^m, m < N (FP64 sincospi), since
 // W_{Ns R}^{r k} = W_N^{r k N / (Ns R)}.
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cstdlib>
-
-#include <type_traits>
 
 #include "gbfft_internal.h"
 #include "mixed_common.cuh"
@@ -29,23 +26,15 @@ namespace gbfft {
 
 // One pass s over the tile: C transforms of length N at src (global when
 // FIRST, else shared memory), written to dst (global when LAST).
-template <int R, bool PAD, typename T>
-__device__ __forceinline__ void mixed_pass(const MixedArgs& a, int s, const T* src, T* dst, bool first, bool last,
-                                           long long col0) {
-  using S = typename Cx<T>::S;
+template <int R, bool PAD>
+__device__ __forceinline__ void mixed_pass(const MixedArgs& a, int s, const double2* src, double2* dst, bool first,
+                                           bool last, long long col0) {
+  using T = double2;
   const T* tw = (const T*)a.tw;
   const int N = a.N;
   const unsigned NB = a.nb[s], nbm = a.nb_m[s], Ns = a.ns[s], nsm = a.ns_m[s];
   const int total = a.C * (int)NB;
   const int stride = (int)a.tws[s];
-  S sx, sy;   // the FP32 kernel reads FP32 copies: no FP64 conversion on its path
-  if constexpr (std::is_same_v<T, double2>) {
-    sx = a.sx;
-    sy = a.sy;
-  } else {
-    sx = a.fsx;
-    sy = a.fsy;
-  }
   for (int b = threadIdx.x; b < total; b += blockDim.x) {
     const int c = (int)fdiv((unsigned)b, nbm), j = b - c * (int)NB;
     const bool ok = col0 + c < a.batch;
@@ -72,7 +61,7 @@ __device__ __forceinline__ void mixed_pass(const MixedArgs& a, int s, const T* s
 #pragma unroll
       for (int q = 0; q < R; ++q) {
         T y = v[q];
-        if (a.scale_out) y = Cx<T>::make(y.x * sx, y.y * sy);
+        if (a.scale_out) y = Cx<T>::make(y.x * a.sx, y.y * a.sy);
         __stcs(dst + m0 + q * (int)Ns, y);
       }
     } else {
@@ -82,8 +71,9 @@ __device__ __forceinline__ void mixed_pass(const MixedArgs& a, int s, const T* s
   }
 }
 
-template <typename T, bool PAD>
-__device__ __forceinline__ void mixed_tile(const MixedArgs& a, T* smem) {
+template <bool PAD>
+__device__ __forceinline__ void mixed_tile(const MixedArgs& a, double2* smem) {
+  using T = double2;
   const long long tile = blockIdx.x;
   const long long col0 = tile * a.C;
   const long long off = col0 * a.N;
@@ -107,21 +97,14 @@ __device__ __forceinline__ void mixed_tile(const MixedArgs& a, T* smem) {
   }
 }
 
-// FP32: two resident CTAs of up to 512 threads (64 registers); FP64: one.
-template <bool PAD>
-__global__ void __launch_bounds__(512, 2) mixed_kernel(const MixedArgs a) {
-  extern __shared__ __align__(16) unsigned char mixed_smem[];
-  mixed_tile<float2, PAD>(a, (float2*)mixed_smem);
-}
 template <bool PAD>
 __global__ void __launch_bounds__(512, 1) mixed_kernel64(const MixedArgs a) {
   extern __shared__ __align__(16) unsigned char mixed_smem[];
-  mixed_tile<double2, PAD>(a, (double2*)mixed_smem);
+  mixed_tile<PAD>(a, (double2*)mixed_smem);
 }
 
-static const void* mixed_fn(bool fp64, bool pad) {
-  return fp64 ? (pad ? (const void*)mixed_kernel64<true> : (const void*)mixed_kernel64<false>)
-              : (pad ? (const void*)mixed_kernel<true> : (const void*)mixed_kernel<false>);
+static const void* mixed_fn(bool pad) {
+  return pad ? (const void*)mixed_kernel64<true> : (const void*)mixed_kernel64<false>;
 }
 
 // Radix schedule: radix-16 passes for 2^a and one 8/4/2 pass for the rest of
@@ -174,66 +157,47 @@ bool mixed_schedule(MixedArgs& a, long long N) {
   return true;
 }
 
+// FP32: the tile kernel of mixr.cuh.
+static int mixr_plan_one_pass(fft_plan* p) {
+  MixrLaunch& L = p->mr[0];
+  int rc = mixr_init(L, p->n, p->batch, 1, nullptr);
+  if (rc) return rc;
+  const size_t tw_bytes = (mixr_table_entries(L.a) * 8 + 255) & ~(size_t)255;
+  if (cudaMalloc(&p->d_tables, tw_bytes + 256) != cudaSuccess) return FFT_ERR_ALLOC;
+  p->d_status = (int*)((char*)p->d_tables + tw_bytes);
+  if (cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess) return FFT_ERR_CUDA;
+  rc = mixr_fill_tables(L, (float2*)p->d_tables, 0);
+  if (rc) return rc;
+  if (cudaStreamSynchronize(0) != cudaSuccess) return FFT_ERR_CUDA;
+  p->launches = 1;
+  return FFT_OK;
+}
+
 int mixed_plan_init(fft_plan* p) {
   MixedArgs& a = p->mixed;
   const long long N = p->n;
   const bool fp64 = p->prec == FFT_PREC_FP64;
+  p->mixed_ct = fp64 ? nullptr : mixed_ct_lookup(N);
+  if (!fp64 && !p->mixed_ct) return mixr_plan_one_pass(p);
   const size_t esz = fp64 ? 16 : 8;
-  // points per CTA when several transforms share one, and the CTA size for
-  // such tiles (in the test build of the library, GBFFT_MIXED_TILE /
-  // GBFFT_MIXED_THREADS override the FP32 values for measurement)
-  long long tile = fp64 ? 2048 : 4096;
-  int small_threads = 256;
-#ifdef GBFFT_TEST_HOOKS
-  if (!fp64) {
-    const char* et = getenv("GBFFT_MIXED_TILE");
-    const char* eh = getenv("GBFFT_MIXED_THREADS");
-    const long long t = (et && *et) ? atoll(et) : 0;
-    const int h = (eh && *eh) ? atoi(eh) : 0;
-    if (t >= 256 && t <= 8192) tile = t;
-    if (h == 128 || h == 256 || h == 512) small_threads = h;
-  }
-#endif
+  constexpr long long tile = 2048;   // points per CTA when several FP64 transforms share one
   if (!mixed_schedule(a, N) || N > (fp64 ? kMixedMaxN64 : kMixedMaxN)) return FFT_ERR_UNSUPPORTED;
-  a.C = N <= tile ? (int)(tile / N) : 1;
+  a.C = p->mixed_ct ? p->mixed_ct->C : N <= tile ? (int)(tile / N) : 1;
   if (a.C > p->batch) a.C = (int)p->batch;
   a.batch = p->batch;
-  p->mixed_threads = a.C * N <= tile ? small_threads : 512;
-  // lengths with a compiled three-pass schedule of composite radices
-  // (mixed_ct.cu): their own tile size, CTA size and padding choice
-  p->mixed_ct = fp64 ? nullptr : mixed_ct_lookup(N);
-  const int generic_C = a.C;
-  if (p->mixed_ct) {
-    a.C = (int)std::min<long long>(p->mixed_ct->C, p->batch);
-    const size_t pts = (size_t)a.C * (size_t)N;
-    const size_t buf = p->mixed_ct->pad ? pts + ((pts - 1) >> 4) + 1 : pts;
-    p->mixed_threads = p->mixed_ct->threads;
-    p->mixed_smem = (int)(2 * buf * esz);
-    if (p->mixed_smem > 227 * 1024) {
-      p->mixed_ct = nullptr;   // does not fit: the run-time schedule below
-      a.C = generic_C;
-      p->mixed_threads = a.C * N <= tile ? small_threads : 512;
-    } else if (p->mixed_smem > 48 * 1024 &&
-               cudaFuncSetAttribute(p->mixed_ct->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->mixed_smem) !=
-                   cudaSuccess) {
-      return FFT_ERR_UNSUPPORTED;
-    }
-  }
+  p->mixed_threads = p->mixed_ct ? p->mixed_ct->threads : a.C * N <= tile ? 256 : 512;
   // padding pays when a radix-8 or -16 pass leads (its writes are strided by
-  // the radix); pure odd-radix lengths keep the unpadded layout
-  // (when the padded buffers fit in shared memory)
+  // the radix) and the padded buffers fit; pure odd-radix lengths keep the
+  // unpadded layout
   const size_t pts = (size_t)a.C * (size_t)N;
   const size_t padded = pts + ((pts - 1) >> 4) + 1;
-  p->mixed_pad = (a.rad[0] >= 8 && 2 * padded * esz <= 227 * 1024) ? 1 : 0;
-  if (!p->mixed_ct) {
-    const size_t buf = p->mixed_pad ? padded : pts;
-    p->mixed_smem = (int)(2 * buf * esz);
-    if (p->mixed_smem > 227 * 1024) return FFT_ERR_UNSUPPORTED;
-    const void* fn = mixed_fn(fp64, p->mixed_pad);
-    if (p->mixed_smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->mixed_smem) != cudaSuccess)
-      return FFT_ERR_UNSUPPORTED;
-  }
+  p->mixed_pad = p->mixed_ct ? p->mixed_ct->pad : (a.rad[0] >= 8 && 2 * padded * esz <= 227 * 1024);
+  p->mixed_smem = (int)(2 * (p->mixed_pad ? padded : pts) * esz);
+  if (p->mixed_smem > 227 * 1024) return FFT_ERR_UNSUPPORTED;
+  const void* fn = p->mixed_ct ? p->mixed_ct->fn : mixed_fn(p->mixed_pad);
+  if (p->mixed_smem > 48 * 1024 &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->mixed_smem) != cudaSuccess)
+    return FFT_ERR_UNSUPPORTED;
   const size_t tw_bytes = ((size_t)N * esz + 255) & ~(size_t)255;
   if (cudaMalloc(&p->d_tables, tw_bytes + 256) != cudaSuccess) return FFT_ERR_ALLOC;
   a.tw = p->d_tables;
@@ -252,6 +216,8 @@ int mixed_exec(fft_plan* p, const void* in, void* out, int conj, double sx, doub
   // in == out is safe: a tile's first pass reads all of it (into shared
   // memory, or into one thread's registers when N is a single radix) before
   // its last pass writes
+  if (p->prec == FFT_PREC_FP32 && !p->mixed_ct)
+    return mixr_launch(p->mr[0], (const float2*)in, (float2*)out, conj, (float)sx, (float)sy, scale_out, s);
   MixedArgs a = p->mixed;
   a.in = in;
   a.out = out;
@@ -264,7 +230,7 @@ int mixed_exec(fft_plan* p, const void* in, void* out, int conj, double sx, doub
   const long long tiles = (p->batch + a.C - 1) / a.C;
   if (tiles > 0x7fffffffLL) return FFT_ERR_UNSUPPORTED;
   void* args[] = {(void*)&a};
-  const void* fn = p->mixed_ct ? p->mixed_ct->fn : mixed_fn(p->prec == FFT_PREC_FP64, p->mixed_pad);
+  const void* fn = p->mixed_ct ? p->mixed_ct->fn : mixed_fn(p->mixed_pad);
   return cudaLaunchKernel(fn, dim3((unsigned)tiles), dim3(p->mixed_threads), args, (size_t)p->mixed_smem, s) ==
                  cudaSuccess
              ? FFT_OK

@@ -1,5 +1,5 @@
-// mixed4.cu -- plans of strided mixed-radix passes (kernels in mixed4.cuh,
-// mixed4_f32.cu, mixed4_f64.cu):
+// mixed4.cu -- plans of two mixed-radix passes (kernels: FP32 mixr.cuh, FP64
+// mixed4.cuh):
 //  * 1-D lengths beyond one on-chip pass: FP64 (complex128) N > 7168 and FP32
 //    7-smooth N > 14336 that are not powers of two.  Sec. 2.3.2's partition:
 //    N = N1 N2, n = n1 N2 + n2, k = k1 + N1 k2,
@@ -19,13 +19,6 @@
 
 namespace gbfft {
 
-const void* mixed4_kernel_fn32(int csh, bool pad);
-const void* mixed4_kernel_fn64(int csh, bool pad);
-
-const void* mixed4_kernel_fn(bool fp64, int csh, bool pad) {
-  return fp64 ? mixed4_kernel_fn64(csh, pad) : mixed4_kernel_fn32(csh, pad);
-}
-
 constexpr int kMixed4Threads = 256;
 constexpr size_t kMixed4SmemLimit = 227 * 1024;
 
@@ -34,33 +27,26 @@ static size_t m4_smem(long long L, int csh, bool pad, size_t esz) {
   return 2 * rows * ((size_t)1 << csh) * esz;
 }
 
-// One pass: sub-length L, ncols columns in each of `batches` batches, element
+// One FP64 pass: sub-length L, ncols columns in each of `batches` batches, element
 // n of column col of batch b at b*bs + col*cs + n*ns on either side.  Columns
-// per CTA: as many as make a tile of about 4096 (FP32) or 2048 (FP64) points,
-// at most 16 (8) and at most ncols, fewer when the buffers do not fit.
+// per CTA: as many as make a tile of about 2048 points, at most 8 and at most ncols, fewer when the buffers do not fit.
 static int m4_pass_init(fft_plan* p, Mixed4Pass& P, long long L, long long ncols, long long batches,
                         long long in_bs, long long in_cs, long long in_ns, long long out_bs, long long out_cs,
                         long long out_ns, const void* tw, int in_role, int out_role) {
-  const bool fp64 = p->prec == FFT_PREC_FP64;
-  const size_t esz = fp64 ? 16 : 8;
+  constexpr size_t esz = 16;
   memset(&P, 0, sizeof(P));
   Mixed4Args& a = P.a;
   if (!mixed_schedule(a.m, L)) return FFT_ERR_UNSUPPORTED;
   a.m.tw = tw;
-  // FP32 sub-lengths with a compiled schedule take it when the batch has
-  // at least its columns per CTA
-  const Mixed4CtInfo* ct = fp64 ? nullptr : mixed4_ct_lookup(L);
-  if (ct && (1LL << ct->csh) > ncols) ct = nullptr;
-  const long long target = fp64 ? 2048 : 4096;
-  const int csh_max = fp64 ? 3 : 4;
+  constexpr long long target = 2048;
+  constexpr int csh_max = 3;
   int csh = 0;
   while (csh < csh_max && (L << (csh + 1)) <= target && (2LL << csh) <= ncols) ++csh;
   while (csh > 0 && m4_smem(L, csh, true, esz) > kMixed4SmemLimit) --csh;
-  if (ct) csh = ct->csh;
   const bool pad = m4_smem(L, csh, true, esz) <= kMixed4SmemLimit;
   const size_t smem = m4_smem(L, csh, pad, esz);
-  if (smem > kMixed4SmemLimit || (ct && !pad)) return FFT_ERR_UNSUPPORTED;
-  P.fn = ct ? ct->fn : mixed4_kernel_fn(fp64, csh, pad);
+  if (smem > kMixed4SmemLimit) return FFT_ERR_UNSUPPORTED;
+  P.fn = mixed4_kernel_fn64(csh, pad);
   if (!P.fn) return FFT_ERR_UNSUPPORTED;
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(P.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
@@ -94,17 +80,16 @@ static int m4_pass_init(fft_plan* p, Mixed4Pass& P, long long L, long long ncols
 
 static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// The twiddle tables of a plan in one allocation: W_La^m (m < La), W_Lb^m
+// The twiddle tables of an FP64 plan in one allocation: W_La^m (m < La), W_Lb^m
 // (m < Lb; shared when La == Lb), and for a four-step plan the two levels
 // of W_N^e, e < N: lo[i] = W_N^i (i < 2^s), hi[j] = W_N^{j 2^s}; then the
-// status word.  Entries are FP64 sincospi values (rounded once for FP32).
+// status word.  Entries are FP64 sincospi values.
 struct M4Tables {
   const void *wa, *wb, *lo, *hi;
   int s;
 };
 static int m4_tables(fft_plan* p, long long La, long long Lb, long long Nft, M4Tables* t) {
-  const bool fp64 = p->prec == FFT_PREC_FP64;
-  const size_t esz = fp64 ? 16 : 8;
+  constexpr size_t esz = 16;
   int s = 0;
   long long nlo = 0, nhi = 0;
   if (Nft > 0) {
@@ -126,35 +111,119 @@ static int m4_tables(fft_plan* p, long long La, long long Lb, long long Nft, M4T
   t->hi = Nft > 0 ? base + ohi : nullptr;
   t->s = s;
   p->d_status = (int*)(base + ost);
-  cudaError_t e = launch_gen_twiddles_step(base + oa, fp64, La, La, 1, 0);
-  if (e == cudaSuccess && Lb != La) e = launch_gen_twiddles_step(base + ob, fp64, Lb, Lb, 1, 0);
-  if (e == cudaSuccess && Nft > 0) e = launch_gen_twiddles_step(base + olo, fp64, Nft, nlo, 1, 0);
-  if (e == cudaSuccess && Nft > 0) e = launch_gen_twiddles_step(base + ohi, fp64, Nft, nhi, nlo, 0);
+  cudaError_t e = launch_gen_twiddles_step(base + oa, true, La, La, 1, 0);
+  if (e == cudaSuccess && Lb != La) e = launch_gen_twiddles_step(base + ob, true, Lb, Lb, 1, 0);
+  if (e == cudaSuccess && Nft > 0) e = launch_gen_twiddles_step(base + olo, true, Nft, nlo, 1, 0);
+  if (e == cudaSuccess && Nft > 0) e = launch_gen_twiddles_step(base + ohi, true, Nft, nhi, nlo, 0);
   if (e != cudaSuccess || cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess ||
       cudaStreamSynchronize(0) != cudaSuccess)
     return FFT_ERR_CUDA;
   return FFT_OK;
 }
 
-// N = N1 N2 with N1 the largest divisor of N at most sqrt(N) whose cofactor
-// is one on-chip sub-transform; in FP32 the largest such N1 for which both
-// lengths have a compiled schedule, when there is one.
+// FP32: N = N1 N2 with the split of the least modelled cost, both passes on
+// the tile kernel of mixr.cuh.
+static int mixr_plan_1d(fft_plan* p) {
+  const long long N = p->n;
+  long long b1 = 0;
+  float best = 0;
+  // factors within 8 : 1 of each other unless there are none
+  for (int wide = 0; wide < 2 && b1 == 0; ++wide) {
+    for (long long d = 2; d * d <= N; ++d) {
+      if (N % d || N / d > kMixedMaxN || (!wide && N / d > 8 * d)) continue;
+      for (const long long n1 : {d, N / d}) {
+        const float ca = mixr_strided_cost(n1, N / n1, p->batch, false);
+        const float cb = mixr_strided_cost(N / n1, n1, p->batch, true);
+        if (ca < 0 || cb < 0) continue;
+        if (b1 == 0 || ca + cb < best) {
+          b1 = n1;
+          best = ca + cb;
+        }
+      }
+    }
+  }
+  if (b1 == 0) return FFT_ERR_UNSUPPORTED;
+  const long long n2 = N / b1;
+  const MixrLayout la = {N, 1, n2, N, 1, n2}, lb = {N, n2, 1, N, 1, b1};
+  int rc = mixr_init(p->mr[0], b1, n2, p->batch, &la);
+  if (!rc) rc = mixr_init(p->mr[1], n2, b1, p->batch, &lb);
+  if (rc) return rc;
+  p->kind = KIND_MIXED_PASSES;
+  p->m4_n1 = b1;
+  p->m4_n2 = N / b1;
+  // the dense twiddle table of the column pass's outputs while it stays small
+  // beside L2, else two levels
+  const bool dense = N <= (1LL << 20);
+  int s = 0;
+  if (!dense) {
+    int bits = 0;
+    while ((1LL << bits) < N) ++bits;
+    s = (bits + 1) / 2;
+  }
+  const long long nlo = dense ? N : 1LL << s, nhi = dense ? 0 : ((N - 1) >> s) + 1;
+  const size_t ob = al256(mixr_table_entries(p->mr[0].a) * 8);
+  const size_t olo = ob + al256(mixr_table_entries(p->mr[1].a) * 8);
+  const size_t ohi = olo + al256(nlo * 8), ost = ohi + al256(nhi * 8);
+  if (cudaMalloc(&p->d_tables, ost + 256) != cudaSuccess) return FFT_ERR_ALLOC;
+  char* base = (char*)p->d_tables;
+  p->d_status = (int*)(base + ost);
+  if (cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess) return FFT_ERR_CUDA;
+  rc = mixr_fill_tables(p->mr[0], (float2*)base, 0);
+  if (!rc) rc = mixr_fill_tables(p->mr[1], (float2*)(base + ob), 0);
+  if (rc) return rc;
+  MixrArgs& a = p->mr[0].a;
+  cudaError_t e;
+  if (dense) {
+    a.ft = (const float2*)(base + olo);
+    a.ft_cols = (unsigned)p->m4_n2;
+    e = launch_gen_four_step((float2*)(base + olo), N, (int)b1, (int)p->m4_n2, 0);
+  } else {
+    a.ft_lo = (const float2*)(base + olo);
+    a.ft_hi = (const float2*)(base + ohi);
+    a.ft_s = s;
+    e = launch_gen_twiddles_step(base + olo, false, N, nlo, 1, 0);
+    if (e == cudaSuccess) e = launch_gen_twiddles_step(base + ohi, false, N, nhi, nlo, 0);
+  }
+  if (e != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess) return FFT_ERR_CUDA;
+  p->ws_bytes = (size_t)N * (size_t)p->batch * 8;
+  p->launches = 2;
+  return FFT_OK;
+}
+
+// FP32 images: contiguous rows, then columns in place in the output.
+static int mixr_plan_2d(fft_plan* p) {
+  const long long ny = p->ny, nx = p->nx, img = ny * nx;
+  const MixrLayout lc = {img, 1, nx, img, 1, nx};
+  int rc = mixr_init(p->mr[0], nx, ny * p->batch, 1, nullptr);
+  if (!rc) rc = mixr_init(p->mr[1], ny, nx, p->batch, &lc);
+  if (rc) return rc;
+  p->kind = KIND_MIXED_PASSES;
+  p->m4_n1 = ny;
+  p->m4_n2 = nx;
+  const size_t ob = al256(mixr_table_entries(p->mr[0].a) * 8), ost = ob + al256(mixr_table_entries(p->mr[1].a) * 8);
+  if (cudaMalloc(&p->d_tables, ost + 256) != cudaSuccess) return FFT_ERR_ALLOC;
+  char* base = (char*)p->d_tables;
+  p->d_status = (int*)(base + ost);
+  if (cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess) return FFT_ERR_CUDA;
+  rc = mixr_fill_tables(p->mr[0], (float2*)base, 0);
+  if (!rc) rc = mixr_fill_tables(p->mr[1], (float2*)(base + ob), 0);
+  if (rc) return rc;
+  if (cudaStreamSynchronize(0) != cudaSuccess) return FFT_ERR_CUDA;
+  p->ws_bytes = 0;
+  p->launches = 2;
+  return FFT_OK;
+}
+
+// FP64: N = N1 N2 with N1 the largest divisor of N at most sqrt(N) whose
+// cofactor is one on-chip sub-transform.
 int mixed4_plan_1d(fft_plan* p) {
-  const bool fp64 = p->prec == FFT_PREC_FP64;
-  const long long N = p->n, Lmax = fp64 ? kMixedMaxN64 : kMixedMaxN;
-  long long n1 = 0, n1_ct = 0;
+  if (p->prec == FFT_PREC_FP32) return mixr_plan_1d(p);
+  const long long N = p->n;
+  long long n1 = 0;
   long long d = (long long)std::sqrt((double)N) + 1;
   while (d * d > N) --d;
-  for (; d >= 2; --d) {
-    if (N % d != 0 || N / d > Lmax) continue;
-    if (n1 == 0) n1 = d;
-    if (!fp64 && mixed4_ct_lookup(d) && mixed4_ct_lookup(N / d)) {
-      n1_ct = d;
-      break;
-    }
-    if (fp64) break;
-  }
-  if (n1_ct) n1 = n1_ct;
+  for (; d >= 2 && n1 == 0; --d)
+    if (N % d == 0 && N / d <= kMixedMaxN64) n1 = d;
   if (n1 == 0) return FFT_ERR_UNSUPPORTED;
   const long long n2 = N / n1;
   M4Tables t;
@@ -173,7 +242,7 @@ int mixed4_plan_1d(fft_plan* p) {
   // row pass: C adjacent k1, the length-N2 transform over n2, to X[k1 + N1 k2]
   rc = m4_pass_init(p, p->m4[1], n2, n1, p->batch, N, n2, 1, N, 1, n1, t.wb, 2, 1);
   if (rc) return rc;
-  p->ws_bytes = (size_t)N * (size_t)p->batch * (fp64 ? 16 : 8);
+  p->ws_bytes = (size_t)N * (size_t)p->batch * 16;
   p->launches = 2;
   return FFT_OK;
 }
@@ -181,6 +250,7 @@ int mixed4_plan_1d(fft_plan* p) {
 // ny-by-nx images: row transforms (input -> output), then column transforms in
 // place in the output.
 int mixed4_plan_2d(fft_plan* p) {
+  if (p->prec == FFT_PREC_FP32) return mixr_plan_2d(p);
   const long long ny = p->ny, nx = p->nx, img = ny * nx;
   M4Tables t;
   int rc = m4_tables(p, nx, ny, 0, &t);
@@ -200,6 +270,14 @@ int mixed4_plan_2d(fft_plan* p) {
 
 int mixed4_exec(fft_plan* p, const void* in, void* out, int conj, double sx, double sy, int scale_out,
                 cudaStream_t s) {
+  if (p->prec == FFT_PREC_FP32) {
+    const bool two_d = p->ws_bytes == 0;
+    if (!two_d && !p->ws) return FFT_ERR_NO_WORKSPACE;
+    float2* mid = two_d ? (float2*)out : (float2*)p->ws;
+    const int rc = mixr_launch(p->mr[0], (const float2*)in, mid, conj, 1.f, 1.f, 0, s);
+    if (rc) return rc;
+    return mixr_launch(p->mr[1], mid, (float2*)out, 0, (float)sx, (float)sy, scale_out, s);
+  }
   void* bufs[3] = {(void*)in, out, p->ws};
   for (int i = 0; i < p->m4n; ++i)
     if ((p->m4[i].in_role == 2 || p->m4[i].out_role == 2) && !p->ws) return FFT_ERR_NO_WORKSPACE;

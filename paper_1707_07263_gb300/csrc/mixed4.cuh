@@ -1,4 +1,4 @@
-// mixed4.cuh -- one strided pass of the mixed-radix recurrence: a tile of
+// mixed4.cuh -- one strided pass of the FP64 mixed-radix recurrence: a tile of
 // C = 2^CSH adjacent sub-transforms ("columns") of length L = a.m.N, element n
 // of column c read from in + b*in_bs + (col0 + c)*in_cs + n*in_ns and written
 // (transformed) to the same form of address in out.
@@ -22,31 +22,22 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include <type_traits>
-
 #include "gbfft_internal.h"
 #include "mixed_common.cuh"
 
 namespace gbfft {
 
-template <int R, int CSH, bool PAD, typename T>
-__device__ __forceinline__ void m4_pass(const Mixed4Args& a, int s, const T* gin, const T* src, T* dst, T* gout,
-                                        bool first, bool last, long long col0, int valid) {
-  using S = typename Cx<T>::S;
+template <int R, int CSH, bool PAD>
+__device__ __forceinline__ void m4_pass(const Mixed4Args& a, int s, const double2* gin, const double2* src,
+                                        double2* dst, double2* gout, bool first, bool last, long long col0,
+                                        int valid) {
+  using T = double2;
   constexpr int C = 1 << CSH;
   const MixedArgs& m = a.m;
   const T* tw = (const T*)m.tw;
   const unsigned NB = m.nb[s], Ns = m.ns[s], nsm = m.ns_m[s];
   const int total = (int)NB << CSH;
   const int stride = (int)m.tws[s];
-  S sx, sy;
-  if constexpr (std::is_same_v<T, double2>) {
-    sx = m.sx;
-    sy = m.sy;
-  } else {
-    sx = m.fsx;
-    sy = m.fsy;
-  }
   const T* ft_lo = (const T*)a.ft_lo;
   const T* ft_hi = (const T*)a.ft_hi;
   const unsigned long long ft_mask = (1ULL << a.ft_s) - 1ULL;
@@ -82,7 +73,7 @@ __device__ __forceinline__ void m4_pass(const Mixed4Args& a, int s, const T* gin
           const unsigned long long e = col * (unsigned long long)kk;
           y = gmul(y, gmul(__ldg(ft_lo + (e & ft_mask)), __ldg(ft_hi + (e >> a.ft_s))));
         }
-        if (m.scale_out) y = Cx<T>::make(y.x * sx, y.y * sy);
+        if (m.scale_out) y = Cx<T>::make(y.x * m.sx, y.y * m.sy);
         __stcs(gout + c * a.out_cs + (long long)kk * a.out_ns, y);
       }
     } else {
@@ -96,8 +87,9 @@ __device__ __forceinline__ void m4_pass(const Mixed4Args& a, int s, const T* gin
 // columns from (t mod tiles_per_batch) * C.  The first pass reads the whole
 // tile from global memory before the last pass writes it, so in == out is
 // safe when the passes of different tiles touch disjoint elements.
-template <typename T, int CSH, bool PAD>
-__device__ __forceinline__ void m4_tiles(const Mixed4Args& a, T* smem) {
+template <int CSH, bool PAD>
+__device__ __forceinline__ void m4_tiles(const Mixed4Args& a, double2* smem) {
+  using T = double2;
   constexpr int C = 1 << CSH;
   const MixedArgs& m = a.m;
   T* const buf0 = smem;

@@ -12,7 +12,7 @@ namespace gbfft {
 template <int CSH, bool PAD>
 __global__ void __launch_bounds__(256, 2) mixed4_kernel64(const Mixed4Args a) {
   extern __shared__ __align__(16) unsigned char m4_smem64[];
-  m4_tiles<double2, CSH, PAD>(a, (double2*)m4_smem64);
+  m4_tiles<CSH, PAD>(a, (double2*)m4_smem64);
 }
 
 const void* mixed4_kernel_fn64(int csh, bool pad) {

@@ -1,12 +1,10 @@
 // mixed_common.cuh -- the butterflies shared by the mixed-radix kernels
-// (mixed.cu, run-time radix schedule; mixed_ct.cu, compile-time schedules):
-// complex arithmetic for FP32 and FP64 elements, radix-2/4/8/16 and odd-prime
-// 3/5/7 DFTs, the per-butterfly twiddles, the padded shared-memory index and
+// (FP64: mixed.cu, mixed4.cuh; FP32: mixr.cuh, mixed_ct.cu): complex
+// arithmetic for FP32 and FP64 elements, radix-2/4/8/16 and odd-prime 3/5/7
+// DFTs, the FP64 per-butterfly twiddles, the padded shared-memory index and
 // the reciprocal division.
 #pragma once
 #include <cuda_runtime.h>
-
-#include <type_traits>
 
 #include "fft_common.cuh"
 
@@ -161,45 +159,21 @@ __device__ __forceinline__ void dft_odd(T* v) {
   for (int q = 0; q < R; ++q) v[q] = out[q];
 }
 
-template <int R, typename T>
-__device__ __forceinline__ void dft_any(T* v) {
+template <int R>
+__device__ __forceinline__ void dft_any(double2* v) {
   if constexpr (R == 3 || R == 5 || R == 7)
     dft_odd<R>(v);
-  else if constexpr (std::is_same_v<T, float2>)
-    dft_fwd<R>(v);
   else
     gdft_pow2<R>(v);
 }
 
-// Twiddles w^r, r = 1..R-1, of one butterfly (w = W_N^e, e = k * stride).
-// FP32: the powers w, w^2, w^4, w^8 that the radix needs are loaded from the
-// W_N^m table, the others are products of them (radix 16: 4 loads + 11
-// products instead of 15 loads; radix 5: 2 + 2; radix 7: 3 + 3); measured
-// 2-16 % faster.  FP64: every power is loaded (FP64 products are the scarce
-// resource; the product form measured 5-10 % slower).
-template <int R, typename T>
-__device__ __forceinline__ void mixed_twiddles(T* v, const T* tw, int e) {
-  if constexpr (std::is_same_v<T, double2>) {
-    // FP64 products cost far more than loads on this GPU: load every power
+// v[r] *= w^r, r = 1..R-1, of one FP64 butterfly (w = W_N^e, e = k * stride).
+// Every power is loaded: FP64 products are the scarce resource (building
+// them from a few loaded powers measured 5-10 % slower).
+template <int R>
+__device__ __forceinline__ void mixed_twiddles(double2* v, const double2* tw, int e) {
 #pragma unroll
-    for (int r = 1; r < R; ++r) v[r] = gmul(v[r], __ldg(tw + r * e));
-    return;
-  }
-  T w[R];
-  w[1] = __ldg(tw + e);
-  if constexpr (R >= 3) w[2] = __ldg(tw + 2 * e);
-  if constexpr (R >= 5) w[4] = __ldg(tw + 4 * e);
-  if constexpr (R >= 9) w[8] = __ldg(tw + 8 * e);
-  if constexpr (R >= 4) w[3] = gmul(w[1], w[2]);
-  if constexpr (R >= 6) w[5] = gmul(w[4], w[1]);
-  if constexpr (R >= 7) w[6] = gmul(w[4], w[2]);
-  if constexpr (R >= 8) w[7] = gmul(w[4], w[3]);
-  if constexpr (R >= 16) {
-#pragma unroll
-    for (int r = 1; r < 8; ++r) w[8 + r] = gmul(w[8], w[r]);
-  }
-#pragma unroll
-  for (int r = 1; r < R; ++r) v[r] = gmul(v[r], w[r]);
+  for (int r = 1; r < R; ++r) v[r] = gmul(v[r], __ldg(tw + r * e));
 }
 
 // Shared-memory index of tile element n: padded by one entry every 16 when

@@ -1,24 +1,19 @@
-// mixed_ct.cu -- mixed-radix transforms (N = 2^a 3^b 5^c) with the radix
-// schedule fixed at compile time for common lengths, in three passes of
-// composite register radices.
+// mixed_ct.cu -- mixed-radix transforms (FP32) with everything fixed at
+// compile time -- length, radices, every divisor -- for the common lengths
+// where that still measures faster than the run-time schedules of mixr.cuh
+// (per 2^25 points on GB300, this kernel against that one: 2000 109 against
+// 112 us, 4000 113 against 125, 10000 172 against 185, 12000 168 against 177;
+// the run-time kernel is faster at 1000, 1200, 1500, 2400, 3000, 5000, 6000
+// and 8000).
 //
-// The run-time kernel (mixed.cu) takes one pass per prime factor or radix-16
-// block: N = 1000 = 8*5*5*5 costs four passes, 12000 seven, each a round trip
-// through shared memory plus run-time index divisions.  Sec. 2.1's split
-// holds for any factorisation, so here N = R0 * R1 * R2 with composite
-// radices of 10..25 points kept in registers (a radix R = A * B is itself a
-// Cooley-Tukey split: A-point DFTs, the inner twiddles W_R^{n2 k1} as
-// compile-time constants, B-point DFTs).  Every length below takes three
-// passes, two exchanges through shared memory; N, the radices and every
-// divisor are template parameters, so the index arithmetic folds to
-// multiplications and shifts.
+// Three passes of composite register radices, two exchanges through two
+// shared-memory buffers.
 //
 // Passes follow the same Stockham recurrence as mixed.cu (natural order in
 // and out): butterfly j of a pass with radix R and Ns = the product of the
 // earlier radices reads a[j + r N/R], multiplies by W_{Ns R}^{r (j mod Ns)}
 // (powers of one W_N table entry), runs the R-point DFT and writes
-// b[(j div Ns) Ns R + (j mod Ns) + q Ns].  FP32 only; other lengths, and
-// FP64, take the run-time kernel.
+// b[(j div Ns) Ns R + (j mod Ns) + q Ns].
 #include <cuda_runtime.h>
 
 #include "gbfft_internal.h"
@@ -88,25 +83,19 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 256 ? 2 : 1) mixed_ct_kern
 }
 
 // Compiled schedules, each the fastest of the orders and factorisations
-// measured on GB300 for its length (radix 25 first, then 8 or 16; e.g.
-// N = 1000: [25, 8, 5] 203 us against 312 for [10, 10, 10] and 420 for the
-// run-time kernel's [8, 5, 5, 5], per 2^26 points), the transforms per CTA,
-// C = floor(4096 / N) as for the run-time kernel, and the threads per CTA
-// (512 where one CTA fills an SM's shared memory, 8000 and up: 12000 350 -> 324
-// us; 256 below, where two or three CTAs share an SM).
-// (Tiles chosen instead to spread every pass's butterflies evenly over the
-// threads -- N = 1000: 5 transforms, 3000: 2 -- measured slower: the larger
-// tiles cost resident CTAs.)  The padded layout where the first pass writes at
+// measured on GB300 for its length, the transforms per CTA and the threads per
+// CTA (512 where one CTA fills an SM's shared memory, 256 below, where two or
+// three CTAs share an SM).  The padded layout where the first pass writes at
 // an even stride.
 #define GBFFT_CT(N, R0, R1, R2, C, T) \
   {N, R0, R1, R2, C, T, (R0 % 2 == 0), (const void*)&mixed_ct_kernel<N, R0, R1, R2, (R0 % 2 == 0), T>}
 
 const MixedCtInfo* mixed_ct_lookup(long long N) {
   static const MixedCtInfo tab[] = {
-      GBFFT_CT(1000, 25, 8, 5, 4, 256),    GBFFT_CT(1200, 25, 16, 3, 3, 256),   GBFFT_CT(1500, 25, 12, 5, 2, 256),
-      GBFFT_CT(2000, 25, 16, 5, 2, 256),   GBFFT_CT(2400, 25, 8, 12, 1, 256),   GBFFT_CT(3000, 25, 8, 15, 1, 256),
-      GBFFT_CT(4000, 25, 16, 10, 1, 256),  GBFFT_CT(5000, 25, 8, 25, 1, 256),   GBFFT_CT(6000, 25, 16, 15, 1, 256),
-      GBFFT_CT(8000, 25, 16, 20, 1, 512),  GBFFT_CT(10000, 25, 16, 25, 1, 512), GBFFT_CT(12000, 25, 24, 20, 1, 512),
+      GBFFT_CT(2000, 25, 16, 5, 2, 256),
+      GBFFT_CT(4000, 25, 16, 10, 1, 256),
+      GBFFT_CT(10000, 25, 16, 25, 1, 512),
+      GBFFT_CT(12000, 25, 24, 20, 1, 512),
   };
   for (const MixedCtInfo& t : tab)
     if (t.N == N) return &t;

@@ -1,7 +1,6 @@
-// mixed_ct.cuh -- compile-time radix building blocks of the mixed-radix
-// kernels with fixed schedules (mixed_ct.cu: one on-chip pass per transform;
-// mixed4_ct.cu: the strided passes of the two-pass plans): constant
-// twiddle products, composite register radices of 10..25 points as
+// mixed_ct.cuh -- compile-time radix building blocks of the FP32 mixed-radix
+// kernels (mixr.cuh: schedules chosen at plan time; mixed_ct.cu: lengths fixed
+// at compile time): constant twiddle products, composite register radices of 10..25 points as
 // Cooley-Tukey splits inside the register file, and the per-butterfly twiddles
 // from one W_N table.
 #pragma once
@@ -63,9 +62,9 @@ __device__ __forceinline__ void ct_dft_split(float2* v) {
     for (int n1 = 0; n1 < A; ++n1) x[n2][n1] = v[B * n1 + n2];
 #pragma unroll
   for (int n2 = 0; n2 < B; ++n2) ct_dft<A>(x[n2]);
-  ct_for<1, B>([&](auto n2c) {
+  ct_for<1, B>([&](auto n2c) __attribute__((always_inline)) {
     constexpr int n2 = decltype(n2c)::value;
-    ct_for<1, A>([&](auto k1c) {
+    ct_for<1, A>([&](auto k1c) __attribute__((always_inline)) {
       constexpr int k1 = decltype(k1c)::value;
       x[n2][k1] = mul_wc<R, n2 * k1>(x[n2][k1]);
     });
@@ -87,13 +86,16 @@ template <int R>
 __device__ __forceinline__ void ct_dft(float2* v) {
   if constexpr (R == 2 || R == 4 || R == 8 || R == 16) dft_fwd<R>(v);
   else if constexpr (R == 3 || R == 5 || R == 7) dft_odd<R>(v);
+  else if constexpr (R == 9) ct_dft_split<3, 3>(v);
   else if constexpr (R == 10) ct_dft_split<2, 5>(v);
   else if constexpr (R == 12) ct_dft_split<4, 3>(v);
+  else if constexpr (R == 14) ct_dft_split<2, 7>(v);
   else if constexpr (R == 15) ct_dft_split<3, 5>(v);
   else if constexpr (R == 20) ct_dft_split<4, 5>(v);
+  else if constexpr (R == 21) ct_dft_split<3, 7>(v);
   else if constexpr (R == 24) ct_dft_split<8, 3>(v);
   else {
-    static_assert(R == 25, "compiled radices: 2, 3, 4, 5, 7, 8, 10, 12, 15, 16, 20, 24, 25");
+    static_assert(R == 25, "compiled radices: 2, 3, 4, 5, 7, 8, 9, 10, 12, 14, 15, 16, 20, 21, 24, 25");
     ct_dft_split<5, 5>(v);
   }
 }
@@ -109,7 +111,7 @@ __device__ __forceinline__ void ct_twiddles(float2* v, const float2* tw, int e) 
   float2 w[R];
 #pragma unroll
   for (int p = 1; p < R; p *= 2) w[p] = __ldg(tw + p * e);
-  ct_for<3, R>([&](auto rc) {
+  ct_for<3, R>([&](auto rc) __attribute__((always_inline)) {
     constexpr int r = decltype(rc)::value;
     constexpr int h = ct_hp2(r);
     if constexpr (h != r) w[r] = cmul(w[h], w[r - h]);

@@ -104,6 +104,40 @@ cudaError_t launch_gen_twiddles_step(void* tab, bool fp64, long long N, long lon
   return cudaGetLastError();
 }
 
+// Twiddle basis of one pass of the FP32 mixed-radix tile kernel (mixr.cuh):
+// tab[e * Ns + k] = W_{Ns R}^{2^e k}, k < Ns, every e with 2^e < R.
+__global__ void gen_mixr_twiddles(float2* tab, int R, int Ns, int count) {
+  const long long M = (long long)Ns * R;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+    const int e = i / Ns, k = i - e * Ns;
+    tab[i] = w_entry((long long)k << e, M);
+  }
+}
+
+cudaError_t launch_gen_mixr_twiddles(float2* tab, int R, int Ns, cudaStream_t s) {
+  int rows = 0;
+  while ((1 << rows) < R) ++rows;
+  const int count = rows * Ns;
+  gen_mixr_twiddles<<<(count + 255) / 256, 256, 0, s>>>(tab, R, Ns, count);
+  return cudaGetLastError();
+}
+
+// tab[k * n2 + c] = W_N^{c k}, k < n1, c < n2 (N = n1 n2): the four-step
+// twiddle of every output of a column pass.
+__global__ void gen_four_step(float2* tab, long long N, int n1, int n2) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long k = i / n2, c = i - k * n2;
+    tab[i] = w_entry(k * c, N);
+  }
+}
+
+cudaError_t launch_gen_four_step(float2* tab, long long N, int n1, int n2, cudaStream_t s) {
+  const long long blocks = (N + 255) / 256;
+  gen_four_step<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(tab, N, n1, n2);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_gen_stage_twiddles(float2* tab, int lg, cudaStream_t s, bool rev, int lgm) {
   const int total = stage_tw_size(lg, rev, lgm);
   if (total == 0) return cudaSuccess;
