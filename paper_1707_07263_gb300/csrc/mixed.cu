@@ -195,8 +195,10 @@ int mixed_plan_init(fft_plan* p) {
   p->mixed_smem = (int)(2 * (p->mixed_pad ? padded : pts) * esz);
   if (p->mixed_smem > 227 * 1024) return FFT_ERR_UNSUPPORTED;
   const void* fn = p->mixed_ct ? p->mixed_ct->fn : mixed_fn(p->mixed_pad);
+  // the limit is a property of the kernel, which plans of other lengths share:
+  // always the largest, or a later plan would lower it under an earlier one
   if (p->mixed_smem > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->mixed_smem) != cudaSuccess)
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
     return FFT_ERR_UNSUPPORTED;
   const size_t tw_bytes = ((size_t)N * esz + 255) & ~(size_t)255;
   if (cudaMalloc(&p->d_tables, tw_bytes + 256) != cudaSuccess) return FFT_ERR_ALLOC;

@@ -48,8 +48,9 @@ static int m4_pass_init(fft_plan* p, Mixed4Pass& P, long long L, long long ncols
   if (smem > kMixed4SmemLimit) return FFT_ERR_UNSUPPORTED;
   P.fn = mixed4_kernel_fn64(csh, pad);
   if (!P.fn) return FFT_ERR_UNSUPPORTED;
+  // (the kernel's limit, which other plans share: always the largest)
   if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(P.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      cudaFuncSetAttribute(P.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixed4SmemLimit) != cudaSuccess)
     return FFT_ERR_CUDA;
   const int C = 1 << csh;
   a.m.C = C;
