@@ -1,0 +1,6 @@
+// fx64_01.cu -- instance of the FP64 tile kernel: contiguous transforms, evenly spaced tile.
+#include "fx64.cuh"
+
+namespace gbfft {
+const void* fx_fn_0_1() { return (const void*)fx_kernel<false, true>; }
+}  // namespace gbfft

@@ -1,0 +1,6 @@
+// fx64_11.cu -- instance of the FP64 tile kernel: strided columns, evenly spaced tile.
+#include "fx64.cuh"
+
+namespace gbfft {
+const void* fx_fn_1_1() { return (const void*)fx_kernel<true, true>; }
+}  // namespace gbfft

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/gbfft.h"
+#include "fx64_math.h"
 #include "mixr_plan.h"
 #include "tile_fft.cuh"
 
@@ -42,27 +43,18 @@ enum PlanKind {
   KIND_MIXED_PASSES = 6   // strided mixed-radix passes: four-step 1-D or 2-D (mixed4.cu)
 };
 
-// One-pass lengths N = 2^a 3^b 5^c 7^d (mixed.cu): FP64, and the FP32
-// lengths of mixed_ct.cu.
-constexpr int kMixedMaxPasses = 16;
-constexpr long long kMixedMaxN = 14336;   // two shared-memory buffers of N complex values fit
-constexpr long long kMixedMaxN64 = 7168;  // the same for FP64 (complex128) values
+// Lengths N = 2^a 3^b 5^c 7^d (mixed.cu, mixed4.cu): the largest of one on-chip pass.
+constexpr long long kMixedMaxN = 14336;
+constexpr long long kMixedMaxN64 = 7168;
+// One launch of a compiled schedule (mixed_ct.cu).
 struct MixedArgs {
-  const void* in;     // float2 (FP32) or double2 (FP64) elements
+  const void* in;
   void* out;
-  const void* tw;     // W_N^m, m < N, same element type
+  const void* tw;     // W_N^m, m < N
   int N, C;           // length; transforms per CTA
   long long batch;
-  int nrad;
-  int rad[kMixedMaxPasses];
-  // per pass: N/R and Ns with their reciprocals ceil(2^32 / d) (0 for d = 1):
-  // q = umulhi(n, m) is exact for n * d < 2^32, which every index here meets
-  unsigned nb[kMixedMaxPasses], nb_m[kMixedMaxPasses];
-  unsigned ns[kMixedMaxPasses], ns_m[kMixedMaxPasses];
-  unsigned tws[kMixedMaxPasses];   // per pass: twiddle stride N / (Ns R) into W_N^m
   int conj_in, scale_out;
-  double sx, sy;      // output scale (1/N of Eq. 2 exact to FP64 for the FP64 kernel)
-  float fsx, fsy;     // the same rounded to FP32 for the FP32 kernel
+  float fsx, fsy;     // output scale
 };
 // One launch of the FP32 mixed-radix tile kernel (mixr.cuh).
 struct MixrArgs {
@@ -103,12 +95,56 @@ struct MixrLayout {
 };
 size_t mixr_table_entries(const MixrArgs& a);
 int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, const MixrLayout* lay);
-float mixr_strided_cost(long long N, long long ncols, long long batches, bool in_rows);
 int mixr_fill_tables(MixrLaunch& L, float2* tab, cudaStream_t s);
 int mixr_launch(const MixrLaunch& L, const float2* in, float2* out, int conj, float sx, float sy, int scale_out,
                 cudaStream_t s);
 cudaError_t launch_gen_mixr_twiddles(float2* tab, int R, int Ns, cudaStream_t s);
 cudaError_t launch_gen_four_step(float2* tab, long long N, int n1, int n2, cudaStream_t s);
+
+// One launch of the FP64 tile kernel (fx64.cuh), laid out as MixrArgs.
+struct FxArgs {
+  const double2* in;
+  double2* out;
+  const int4* tw;              // Q62 twiddles of every pass, pass s at tw_off[s]: (r - 1) Ns + k
+  const int4* wn;              // W_N^m, m < N (tiles with an infinity or a NaN)
+  int N, C;
+  int csh, pitch, in_rows;
+  int pad_sh, slot_off;        // one pad entry every 2^pad_sh; byte offset of the exponent slots
+  int nrad;
+  int rad[mixr::kMaxPasses], head[mixr::kMaxPasses];   // radix and its headroom bits
+  unsigned nb[mixr::kMaxPasses], nb_m[mixr::kMaxPasses];
+  unsigned ns[mixr::kMaxPasses], ns_m[mixr::kMaxPasses];
+  int ld_st[mixr::kMaxPasses], st_st[mixr::kMaxPasses];   // tile strides of a butterfly's inputs and outputs
+  unsigned tw_off[mixr::kMaxPasses];
+  long long ncols;
+  long long tile0;
+  long long tiles_per_batch, in_bs, out_bs;
+  unsigned in_cs, in_ns, out_cs, out_ns;
+  const int4* ft;              // four-step twiddles, dense or in two levels
+  unsigned ft_cols;
+  const int4* ft_lo;
+  const int4* ft_hi;
+  int ft_s;
+  int conj_in, conj_out;
+  // output scale: times 2^scale_ex, and scale_q (times 1/4) unless it is a power of two
+  int scale_ex;
+  Q62 scale_q;
+  double scale;                // the same in FP64
+};
+struct FxLaunch {
+  FxArgs a;
+  const void* fn;
+  int threads, smem;
+  long long ntiles;
+};
+size_t fx_table_entries(const FxArgs& a);
+int fx_init(FxLaunch& L, long long N, long long ncols, long long batches, const MixrLayout* lay);
+int fx_fill_tables(FxLaunch& L, int4* tab, cudaStream_t s);
+int fx_launch(const FxLaunch& L, const double2* in, double2* out, int conj_in, int conj_out, double scale,
+              cudaStream_t s);
+cudaError_t launch_gen_fx_twiddles(int4* tab, int R, int Ns, cudaStream_t s);
+cudaError_t launch_gen_fx_power(int4* tab, long long N, long long count, long long step, cudaStream_t s);
+cudaError_t launch_gen_fx_four_step(int4* tab, long long N, int n1, int n2, cudaStream_t s);
 
 // Mixed-radix lengths with a compile-time three-pass schedule (mixed_ct.cu).
 struct MixedCtInfo {
@@ -121,37 +157,7 @@ struct MixedCtInfo {
 };
 const MixedCtInfo* mixed_ct_lookup(long long N);
 
-int mixed_radices(long long N, int* rad);
-bool mixed_schedule(MixedArgs& a, long long N);
 int mixed_plan_init(fft_plan* p);
-
-// Strided passes of the mixed-radix recurrence (mixed4.cu): a batch of
-// sub-transforms of length m.N ("columns") whose element n sits at
-// col * cs + n * ns from the batch's base, C = 2^csh adjacent columns per
-// CTA.  Two such passes make the four-step split of a length beyond one
-// on-chip pass (the column pass multiplies its output by W_Nt^{col * k}) and
-// the rows-then-columns 2-D transform.
-struct Mixed4Args {
-  MixedArgs m;                 // sub-length schedule, W_{m.N} table, in/out, conj and output scale
-  long long in_bs, out_bs;     // element offset of batch b: b * bs
-  long long in_cs, in_ns, out_cs, out_ns;
-  long long ncols;             // columns per batch
-  long long tiles_per_batch;   // ceil(ncols / C)
-  long long ntiles;            // tiles_per_batch * batches
-  const void* ft_lo;           // four-step twiddle W_Nt^e = ft_lo[e & (2^ft_s - 1)] * ft_hi[e >> ft_s]
-  const void* ft_hi;           // of e = col * k on the output (NULL: none)
-  int ft_s;
-};
-struct Mixed4Pass {
-  Mixed4Args a;
-  const void* fn;
-  int threads, smem;
-  long long grid;
-  int in_role, out_role;       // 0 the caller's input, 1 its output, 2 the workspace
-};
-constexpr int kMixed4MaxPasses = 2;
-// FP64 kernel, 2^csh columns per CTA, padded index
-const void* mixed4_kernel_fn64(int csh, bool pad);
 int mixed4_plan_1d(fft_plan* p);
 int mixed4_plan_2d(fft_plan* p);
 int mixed4_exec(fft_plan* p, const void* in, void* out, int conj, double sx, double sy, int scale_out,
@@ -160,7 +166,6 @@ cudaError_t launch_gen_twiddles_step(void* tab, bool fp64, long long N, long lon
                                      cudaStream_t s);
 int mixed_exec(fft_plan* p, const void* in, void* out, int conj, double sx, double sy, int scale_out,
                cudaStream_t s);
-cudaError_t launch_gen_twiddles_n(float2* tab, long long N, long long count, cudaStream_t s);
 cudaError_t launch_gen_twiddles_n64(double2* tab, long long N, long long count, cudaStream_t s);
 
 cudaError_t launch_gen_stage_twiddles(float2* tab, int lg, cudaStream_t s, bool rev = false, int lgm = 4);
@@ -230,11 +235,10 @@ struct fft_plan {
 
   // mixed-radix plans (KIND_MIXED)
   gbfft::MixedArgs mixed;
-  int mixed_threads, mixed_smem, mixed_pad;
+  int mixed_smem;
   const gbfft::MixedCtInfo* mixed_ct;   // compile-time schedule for this length (FP32), or NULL
   gbfft::MixrLaunch mr[2];   // FP32 mixed radix: one tile pass, or the two passes of a split
-  gbfft::Mixed4Pass m4[gbfft::kMixed4MaxPasses];   // KIND_MIXED_PASSES
-  int m4n;
+  gbfft::FxLaunch fx[2];     // FP64: the same
   long long m4_n1, m4_n2;   // four-step: column length N1, row length N2 (N = N1 N2); 2-D: ny, nx
   const float2* pre_tw;               // its W_N^n table, n < N/2
   long long tma_grid;                 // its resident-CTA grid

@@ -9,8 +9,8 @@
 // Three passes of composite register radices, two exchanges through two
 // shared-memory buffers.
 //
-// Passes follow the same Stockham recurrence as mixed.cu (natural order in
-// and out): butterfly j of a pass with radix R and Ns = the product of the
+// Passes follow the Stockham recurrence of mixr.cuh (natural order in and
+// out): butterfly j of a pass with radix R and Ns = the product of the
 // earlier radices reads a[j + r N/R], multiplies by W_{Ns R}^{r (j mod Ns)}
 // (powers of one W_N table entry), runs the R-point DFT and writes
 // b[(j div Ns) Ns R + (j mod Ns) + q Ns].

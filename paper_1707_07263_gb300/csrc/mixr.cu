@@ -43,22 +43,14 @@ int mixr_fill_tables(MixrLaunch& L, float2* tab, cudaStream_t s) {
   return FFT_OK;
 }
 
-// Modelled cost of a strided pass (to choose between splits of a longer
-// length), negative if there is none.
-float mixr_strided_cost(long long N, long long ncols, long long batches, bool in_rows) {
-  Choice c;
-  if (choose(c, N, ncols, ncols * batches, true, in_rows)) return -1.f;
-  const long long tiles = (ncols + c.C - 1) / c.C;   // the last tile of a batch may be partly empty
-  return c.cost * (float)(tiles * c.C) / (float)ncols + run_cost(c.C, ncols);
-}
-
 // Fills L for `batches` batches of ncols sub-transforms of length N
 // (contiguous when lay is NULL: then batches must be 1).
 int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, const MixrLayout* lay) {
   memset(&L, 0, sizeof(L));
   const bool strided = lay != nullptr, in_rows = lay && lay->in_ns == 1 && lay->in_cs != 1;
   Choice best;
-  const int rc = choose(best, N, ncols, ncols * batches, strided, in_rows);
+  const Family& f = family_f32();
+  const int rc = choose(f, best, N, ncols, ncols * batches, strided, in_rows);
   if (rc) return rc;
   const int* rad = best.q.rad;
   MixrArgs& a = L.a;
@@ -77,7 +69,7 @@ int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, co
     ns *= (unsigned)rad[s];
   }
   a.ncols = ncols;
-  const bool pad = needs_pad(rad[0], strided, in_rows, best.C);
+  const bool pad = needs_pad(f, rad[0], strided, in_rows, best.C);
   if (lay) {
     while ((1 << a.csh) < best.C) ++a.csh;
     a.in_rows = in_rows;
@@ -93,7 +85,7 @@ int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, co
   } else {
     L.ntiles = (ncols + best.C - 1) / best.C;
   }
-  L.smem = a.nrad > 1 ? (int)tile_bytes(N, best.C, strided, in_rows, pad) : 0;
+  L.smem = a.nrad > 1 ? (int)tile_bytes(f, N, best.C, strided, in_rows, pad) : 0;
   L.threads = best.T;
   L.fn = mixr_fn(lay != nullptr, pad, best.big);
   if (L.smem > 48 * 1024 &&

@@ -1,6 +1,6 @@
-// mixr_plan.h -- the plan of one FP32 mixed-radix tile (mixr.cuh): the radix
-// schedule, columns and threads per CTA of a sub-transform of any 7-smooth
-// length, chosen by a cost model of its passes.  Plain C++17, so the host test
+// mixr_plan.h -- the plan of one mixed-radix tile (FP32: mixr.cuh, FP64:
+// fx64.cuh): the radix schedule, columns and threads per CTA of a
+// sub-transform of any 7-smooth length, chosen by a cost model of its passes.  Plain C++17, so the host test
 // suite can check every length's plan with g++.
 #pragma once
 #include <algorithm>
@@ -14,13 +14,21 @@ namespace gbfft {
 namespace mixr {
 
 constexpr int kMaxPasses = 6;
-constexpr int kRadices[] = {2, 3, 4, 5, 7, 8, 9, 10, 12, 14, 15, 16, 20, 21, 24, 25};
-constexpr int kThreads[] = {96, 128, 192, 256, 320, 384};
-constexpr int kThreadsBig[] = {256, 320, 384, 448, 512};
-constexpr int kPoints = 25, kPointsBig = 32;          // middle-pass points a thread may hold
-constexpr long long kMaxTile = 384 * kPoints;         // 9600 points
-constexpr long long kMaxTileBig = 512 * kPointsBig;
 constexpr size_t kSmemLimit = 227 * 1024, kSmemSm = 228 * 1024;
+
+// What the two kernels differ in.
+struct Family {
+  int nradices, radices[16];   // ascending
+  int threads[6], threads_big[6];   // CTA sizes of small and big tiles (0 ends the list)
+  int points, points_big;      // points a thread may hold in a middle pass
+  bool first_held;             // the first pass holds its points too
+  long long max_tile, max_tile_big, big_from;   // tile points; big CTAs above big_from
+  int regs, regs_big;
+  int elem;                    // bytes of a tile element
+  int max_cols;                // strided columns that fill 128 bytes
+  int slot_bytes;              // per pass and column, beside the tile
+  float (*pass_cost)(int r, bool first, bool last, bool pad);
+};
 
 // FP32 instructions a point of the R-point DFT (additions, constant products)
 inline float dft_cost(int r) {
@@ -54,6 +62,43 @@ inline float twiddle_cost(int r) {
   return (2.f * e + 4.f * (r - 1 - e) + 4.f * (r - 1)) / r;
 }
 
+// The passes' arithmetic, index work and exchanges.  The weights (and those of
+// tile_cost) are a fit to 9,000 measured (schedule, columns, threads) of 41
+// lengths from 30 to 12288 on GB300: the pick is 0.7 % (at most 5 %) slower
+// than the fastest measured.
+inline float pass_cost_f32(int r, bool first, bool last, bool pad) {
+  float per = dft_cost(r) + 10.8f / (float)r + (pad ? 1.6f : 0.f);
+  if (!first) per += 1.48f * twiddle_cost(r) + (r >= 15 ? 4.5f : 0.f) + (r >= 20 ? 4.f : 0.f);
+  if (!first && !last) per += 4.5f;
+  return per;
+}
+// 64-bit integer instructions a point: two an addition, about 20 a rotation,
+// 6 a real constant product
+inline float pass_cost_fx(int r, bool first, bool last, bool) {
+  const float dft = r == 2 ? 4.f : r == 3 ? 20.f : r == 4 ? 8.f : r == 5 ? 35.f : r == 7 ? 60.f : r == 8 ? 18.f
+                    : r == 9 ? 52.f : r == 10 ? 48.f : r == 12 ? 42.f : r == 14 ? 73.f : r == 15 ? 70.f : 30.f;
+  return dft + 30.f / (float)r + 10.f + (first ? 20.f : 20.f * (float)(r - 1) / (float)r) + (last ? 25.f : 6.f);
+}
+
+inline const Family& family_f32() {
+  // up to 384 threads of 80 registers (two CTAs of 384, three of 256 or six of
+  // 128 share an SM), 512 of 128 for big tiles
+  static const Family f = {16,
+                           {2, 3, 4, 5, 7, 8, 9, 10, 12, 14, 15, 16, 20, 21, 24, 25},
+                           {96, 128, 192, 256, 320, 384},
+                           {256, 320, 384, 448, 512, 0},
+                           25, 32, false, 9600, 16384, 6144, 80, 128, 8, 16, 0, pass_cost_f32};
+  return f;
+}
+inline const Family& family_fx() {
+  static const Family f = {12,
+                           {2, 3, 4, 5, 7, 8, 9, 10, 12, 14, 15, 16},
+                           {64, 96, 128, 192, 256, 0},
+                           {320, 384, 448, 512, 0, 0},
+                           18, 18, true, 4096, 8192, 2048, 128, 128, 16, 8, 4, pass_cost_fx};
+  return f;
+}
+
 struct Schedule {
   int n, rad[kMaxPasses];
 };
@@ -64,34 +109,27 @@ struct Choice {
   float cost;
 };
 
-inline bool needs_pad(int r0, bool strided, bool in_rows, int C) {
+inline bool needs_pad(const Family& f, int r0, bool strided, bool in_rows, int C) {
   if (r0 & 1) return false;
-  return !strided || in_rows || C < 16;   // 16 columns fill every bank whatever the row stride
+  return !strided || in_rows || C < f.max_cols;   // max_cols columns fill every bank whatever the row stride
 }
-inline size_t tile_bytes(long long N, int C, bool strided, bool in_rows, bool pad) {
+inline size_t tile_bytes(const Family& f, long long N, int C, bool strided, bool in_rows, bool pad) {
   const long long rows = strided ? N : C * N;
   const long long padded = pad ? rows + ((rows - 1) >> 4) : rows;
-  return (size_t)padded * (strided ? C + (in_rows ? 1 : 0) : 1) * 8;
+  return (size_t)padded * (strided ? C + (in_rows ? 1 : 0) : 1) * (size_t)f.elem;
 }
 
-// Cost of a tile, in instructions a point: the passes' arithmetic, index work
-// and exchanges, with part of what a pass's last, partly filled round leaves
-// idle, and more where few warps share an SM.  The weights are a fit to 9,000
-// measured (schedule, columns, threads) of 41 lengths from 30 to 12288 on
-// GB300: the pick is 0.7 % (at most 5 %) slower than the fastest measured.
-inline float tile_cost(const Choice& c, long long N, size_t smem, bool pad) {
+// Cost of a tile, in instructions a point, with part of what a pass's last,
+// partly filled round leaves idle, and more where few warps share an SM.
+inline float tile_cost(const Family& f, const Choice& c, long long N, size_t smem, bool pad) {
   const float P = (float)c.C * (float)N;
   float sum = 0;
   for (int s = 0; s < c.q.n; ++s) {
-    const int r = c.q.rad[s];
-    const float nb = P / (float)r;
+    const float nb = P / (float)c.q.rad[s];
     const float rounds = (float)(int)((nb + (float)c.T - 1.f) / (float)c.T);
-    float per = dft_cost(r) + 10.8f / (float)r + (pad ? 1.6f : 0.f);
-    if (s > 0) per += 1.48f * twiddle_cost(r) + (r >= 15 ? 4.5f : 0.f) + (r >= 20 ? 4.f : 0.f);
-    if (s > 0 && s + 1 < c.q.n) per += 4.5f;
-    sum += per * (1.f + 0.22f * (1.f - nb / (rounds * (float)c.T)));
+    sum += f.pass_cost(c.q.rad[s], s == 0, s + 1 == c.q.n, pad) * (1.f + 0.22f * (1.f - nb / (rounds * (float)c.T)));
   }
-  const int regs = c.big ? 128 : 80;
+  const int regs = c.big ? f.regs_big : f.regs;
   int ctas = std::min<int>(65536 / (regs * c.T), (int)(kSmemSm / (smem + 1024)));
   ctas = std::max(1, std::min(ctas, 32));
   const float warps = (float)(ctas * c.T) / 32.f;
@@ -100,26 +138,30 @@ inline float tile_cost(const Choice& c, long long N, size_t smem, bool pad) {
   return sum * (1.f + 0.094f * (float)c.T / 256.f);
 }
 // Cost of strided global runs of C of the ncols adjacent elements against
-// aligned runs of 16 (128 bytes): shorter runs, and runs that start inside a
+// aligned runs of 128 bytes: shorter runs, and runs that start inside a
 // 32-byte sector or a 128-byte line.
-inline float run_cost(int C, long long ncols) {
-  const float run = C >= 16 ? 0.f : C >= 8 ? 8.f : C >= 4 ? 15.f : C >= 2 ? 80.f : 200.f;
-  return run + (ncols % 4 ? 10.f : ncols % 16 ? 2.f : 0.f);
+inline float run_cost(const Family& f, int C, long long ncols) {
+  const int b = C * f.elem;
+  const float run = b >= 128 ? 0.f : b >= 64 ? 8.f : b >= 32 ? 15.f : b >= 16 ? 80.f : 200.f;
+  const long long step = ncols * f.elem;
+  return run + (step % 32 ? 10.f : step % 128 ? 2.f : 0.f);
 }
 
 // Every ordered factorisation of `rest` into npass register radices.
-inline void factorisations(long long rest, int depth, int npass, Schedule& cur, std::vector<Schedule>& out) {
+inline void factorisations(const Family& f, long long rest, int depth, int npass, Schedule& cur,
+                           std::vector<Schedule>& out) {
   if (depth == npass) {
     if (rest == 1) out.push_back(cur);
     return;
   }
   long long most = 1;   // what the remaining passes can still cover
-  for (int i = depth; i < npass; ++i) most *= 25;
+  for (int i = depth; i < npass; ++i) most *= f.radices[f.nradices - 1];
   if (rest > most) return;
-  for (const int r : kRadices) {
+  for (int i = 0; i < f.nradices; ++i) {
+    const int r = f.radices[i];
     if (rest % r) continue;
     cur.rad[depth] = r;
-    factorisations(rest / r, depth + 1, npass, cur, out);
+    factorisations(f, rest / r, depth + 1, npass, cur, out);
   }
 }
 
@@ -127,22 +169,23 @@ inline void factorisations(long long rest, int depth, int npass, Schedule& cur, 
 // of length N with ncols columns a batch, `total` in all; FFT_ERR_UNSUPPORTED
 // if there is none.  Fewest passes first (lengths above 7 take at least two: a single
 // radix would read and write global memory at a stride of N).
-inline int choose(Choice& best, long long N, long long ncols, long long total, bool strided, bool in_rows) try {
+inline int choose(const Family& f, Choice& best, long long N, long long ncols, long long total, bool strided,
+                  bool in_rows) try {
   memset(&best, 0, sizeof(best));
   std::vector<Schedule> qs;
   for (int np = N > 7 ? 2 : 1; np <= kMaxPasses; ++np) {
     Schedule cur;
     memset(&cur, 0, sizeof(cur));
     cur.n = np;
-    factorisations(N, 0, np, cur, qs);
+    factorisations(f, N, 0, np, cur, qs);
     if (qs.empty()) continue;
-    // columns per CTA.  Strided: the widest power of two up to 16 that the tile
-    // holds.  Contiguous: tiles of 1500 to 9600 points, fewer when the batch
-    // would not give every SM a few CTAs.
-    long long cmax = std::min(std::max(1LL, kMaxTile / N), std::max(1LL, ncols));
+    // columns per CTA.  Strided: the widest power of two that the tile holds, up
+    // to 128 bytes.  Contiguous: tiles of 1500 points to the largest, fewer when
+    // the batch would not give every SM a few CTAs.
+    long long cmax = std::min(std::max(1LL, f.max_tile / N), std::max(1LL, ncols));
     long long cmin = 1;
     if (strided) {
-      cmax = std::min(cmax, 16LL);
+      cmax = std::min<long long>(cmax, f.max_cols);
       while (cmin * 2 <= cmax) cmin *= 2;
     } else {
       cmax = std::min(cmax, std::max(1LL, total / (152 * 4)));
@@ -150,24 +193,26 @@ inline int choose(Choice& best, long long N, long long ncols, long long total, b
     }
     for (long long C = cmin; C <= cmax; C += strided ? cmax : std::max(1LL, C / 8)) {
       for (int big = 0; big < 2; ++big) {
-        if (big && C * N <= 6144) continue;
-        if (C * N > (big ? kMaxTileBig : kMaxTile)) continue;
-        for (int ti = 0; ti < (big ? 5 : 6); ++ti) {
+        if (big && C * N <= f.big_from) continue;
+        if (C * N > (big ? f.max_tile_big : f.max_tile)) continue;
+        for (int ti = 0; ti < 6; ++ti) {
           Choice c;
           c.C = (int)C;
-          c.T = big ? kThreadsBig[ti] : kThreads[ti];
+          c.T = big ? f.threads_big[ti] : f.threads[ti];
           c.big = big != 0;
+          if (c.T == 0) break;
           if (ti > 0 && C * N < 6LL * c.T) continue;
           for (const Schedule& q : qs) {
             bool fits = true;   // a middle pass holds its butterflies in registers
-            for (int s = 1; s + 1 < np; ++s)
-              fits = fits && C * N / q.rad[s] <= (long long)std::max(1, (big ? kPointsBig : kPoints) / q.rad[s]) * c.T;
+            for (int s = f.first_held ? 0 : 1; s + 1 < np; ++s)
+              fits = fits && C * N / q.rad[s] <= (long long)std::max(1, (big ? f.points_big : f.points) / q.rad[s]) * c.T;
             if (!fits) continue;
             c.q = q;
-            const bool pad = needs_pad(q.rad[0], strided, in_rows, c.C);
-            const size_t smem = np > 1 ? tile_bytes(N, c.C, strided, in_rows, pad) : 0;
+            const bool pad = needs_pad(f, q.rad[0], strided, in_rows, c.C);
+            const size_t smem =
+                np > 1 ? tile_bytes(f, N, c.C, strided, in_rows, pad) + (size_t)(f.slot_bytes * np * c.C) : 0;
             if (smem > kSmemLimit) continue;
-            c.cost = tile_cost(c, N, smem, pad);
+            c.cost = tile_cost(f, c, N, smem, pad);
             if (best.q.n == 0 || c.cost < best.cost) best = c;
           }
         }
@@ -179,6 +224,37 @@ inline int choose(Choice& best, long long N, long long ncols, long long total, b
   return FFT_ERR_UNSUPPORTED;
 } catch (...) {   // no exception leaves the C ABI
   return FFT_ERR_ALLOC;
+}
+
+// Modelled cost of a strided pass (to choose between splits of a longer
+// length), negative if there is none.
+inline float strided_cost(const Family& f, long long N, long long ncols, long long batches, bool in_rows) {
+  Choice c;
+  if (choose(f, c, N, ncols, ncols * batches, true, in_rows)) return -1.f;
+  const long long tiles = (ncols + c.C - 1) / c.C;   // the last tile of a batch may be partly empty
+  return c.cost * (float)(tiles * c.C) / (float)ncols + run_cost(f, c.C, ncols);
+}
+
+// N = n1 n2, both at most most: the column length n1 of the split with the
+// least modelled cost of its column and row passes, 0 if there is none.
+inline long long choose_split(const Family& f, long long N, long long batches, long long most) {
+  long long b1 = 0;
+  float best = 0;
+  // factors within 8 : 1 of each other unless there are none
+  for (int wide = 0; wide < 2 && b1 == 0; ++wide)
+    for (long long d = 2; d * d <= N; ++d) {
+      if (N % d || N / d > most || (!wide && N / d > 8 * d)) continue;
+      for (const long long n1 : {d, N / d}) {
+        const float ca = strided_cost(f, n1, N / n1, batches, false);
+        const float cb = strided_cost(f, N / n1, n1, batches, true);
+        if (ca < 0 || cb < 0) continue;
+        if (b1 == 0 || ca + cb < best) {
+          b1 = n1;
+          best = ca + cb;
+        }
+      }
+    }
+  return b1;
 }
 
 }  // namespace mixr

@@ -44,41 +44,9 @@ __global__ void gen_power_twiddles(float2* tab, int lgN, long long count, long l
     tab[i] = w_entry((i * step) % N, N);
 }
 
-// tab[m] = W_N^m, m < count, for any N (mixed-radix lengths).
-__global__ void gen_twiddles_n(float2* tab, long long N, long long count) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x)
-    tab[i] = w_entry(i % N, N);
-}
-
-cudaError_t launch_gen_twiddles_n(float2* tab, long long N, long long count, cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  const long long blocks = (count + 255) / 256;
-  gen_twiddles_n<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(tab, N, count);
-  return cudaGetLastError();
-}
-
-// tab[m] = W_N^m in FP64, m < count (FP64 transforms).
-__global__ void gen_twiddles_n64(double2* tab, long long N, long long count) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x) {
-    double sn, cs;
-    sincospi(-2.0 * (double)(i % N) / (double)N, &sn, &cs);
-    tab[i] = make_double2(cs, sn);
-  }
-}
-
-cudaError_t launch_gen_twiddles_n64(double2* tab, long long N, long long count, cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  const long long blocks = (count + 255) / 256;
-  gen_twiddles_n64<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(tab, N, count);
-  return cudaGetLastError();
-}
-
-// tab[i] = W_N^{(i * step) mod N}, i < count, for any N (the strided
-// mixed-radix plans: sub-length tables with step 1, and the high level of a
-// two-level four-step table with step 2^s); FP64 entries, or rounded once to
-// FP32.
+// tab[i] = W_N^{(i * step) mod N}, i < count, for any N (step 1: one level;
+// the high level of a two-level table: step 2^s); FP64 entries, or rounded
+// once to FP32.
 template <typename T>
 __global__ void gen_twiddles_step(T* tab, long long N, long long count, long long step) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
@@ -135,6 +103,53 @@ __global__ void gen_four_step(float2* tab, long long N, int n1, int n2) {
 cudaError_t launch_gen_four_step(float2* tab, long long N, int n1, int n2, cudaStream_t s) {
   const long long blocks = (N + 255) / 256;
   gen_four_step<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(tab, N, n1, n2);
+  return cudaGetLastError();
+}
+
+// W_M^m as Q62 halves (re low, re high, im low, im high).
+__device__ __forceinline__ int4 w_entry_q62(long long m, long long M) {
+  const FxCosSin w = fx_cossin(m % M, M);
+  const Q62 r = q62_split(w.c), i = q62_split(-w.s);
+  return make_int4(r.l, r.h, i.l, i.h);
+}
+
+// Twiddles of one pass of the FP64 tile kernel (fx64.cuh):
+// tab[(r - 1) Ns + k] = W_{Ns R}^{r k}.
+__global__ void gen_fx_twiddles(int4* tab, int R, int Ns) {
+  const int count = (R - 1) * Ns;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+    const int r = i / Ns, k = i - r * Ns;
+    tab[i] = w_entry_q62((long long)(r + 1) * k, (long long)Ns * R);
+  }
+}
+cudaError_t launch_gen_fx_twiddles(int4* tab, int R, int Ns, cudaStream_t s) {
+  gen_fx_twiddles<<<((R - 1) * Ns + 255) / 256, 256, 0, s>>>(tab, R, Ns);
+  return cudaGetLastError();
+}
+
+// tab[i] = W_N^{i step}, i < count
+__global__ void gen_fx_power(int4* tab, long long N, long long count, long long step) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
+       i += (long long)gridDim.x * blockDim.x)
+    tab[i] = w_entry_q62(i * step, N);
+}
+cudaError_t launch_gen_fx_power(int4* tab, long long N, long long count, long long step, cudaStream_t s) {
+  const long long blocks = (count + 255) / 256;
+  gen_fx_power<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(tab, N, count, step);
+  return cudaGetLastError();
+}
+
+// tab[k n2 + c] = W_N^{c k}, k < n1, c < n2
+__global__ void gen_fx_four_step(int4* tab, long long N, int n2) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long k = i / n2, c = i - k * n2;
+    tab[i] = w_entry_q62(k * c, N);
+  }
+}
+cudaError_t launch_gen_fx_four_step(int4* tab, long long N, int, int n2, cudaStream_t s) {
+  const long long blocks = (N + 255) / 256;
+  gen_fx_four_step<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(tab, N, n2);
   return cudaGetLastError();
 }
 
