@@ -17,5 +17,7 @@ def __getattr__(name):
     if name in ("fft", "ifft", "fft2", "ifft2", "fft_many", "fft_host", "HostPipeline", "range_compress", "rfft", "irfft", "Plan", "get_plan",
                 "clear_plan_cache", "PREC"):
         from . import api
-        return getattr(api, name)
+        value = getattr(api, name)
+        globals()[name] = value   # later uses find it without this function (2.7 us a call)
+        return value
     raise AttributeError(name)

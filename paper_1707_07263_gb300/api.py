@@ -16,6 +16,7 @@ import ctypes
 import threading
 
 import torch
+import torch.autograd.forward_ad as _forward_ad
 
 from . import _lib as L
 
@@ -37,8 +38,19 @@ def _prec_code(prec) -> int:
 
 
 def _stream_handle(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is None:   # the current stream of the current device, without a Stream object (3 us a call)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return int(stream.cuda_stream)
+
+
+def _direct(x: torch.Tensor) -> bool:
+    """Whether a call on x may run without torch.autograd.Function (7 us a
+    call): x needs no gradient and is a plain tensor, and no transform that
+    looks at the Function is active (forward-mode AD, functorch's vmap / grad /
+    jvp, tracing, compilation)."""
+    return (type(x) is torch.Tensor and not (x.requires_grad and torch.is_grad_enabled())
+            and not torch._C._are_functorch_transforms_active() and _forward_ad._current_level < 0
+            and torch._C._get_tracing_state() is None and not torch.compiler.is_compiling())
 
 
 class Plan:
@@ -79,6 +91,7 @@ class Plan:
             if not h:
                 raise L.GbfftError(self.lib.fft_last_error(), f"plan {kind} {shape} batch={batch} prec={prec}")
             self.handle = ctypes.c_void_p(h)
+            self.points = self.numel()
             self.ws_bytes = int(self.lib.fft_plan_workspace_bytes(self.handle))
             self.workspace = None
             if self.ws_bytes:
@@ -105,9 +118,9 @@ class Plan:
 
     def exec_ptr(self, in_ptr: int, out_ptr: int, dir: int | None = None, stream=None) -> None:
         d = self.dir if dir is None else int(dir)
-        rc = self.lib.fft_exec_dir(self.handle, ctypes.c_void_p(in_ptr), ctypes.c_void_p(out_ptr), d,
-                                   ctypes.c_void_p(_stream_handle(stream)))
-        L.check(rc, "fft_exec")
+        rc = self.lib.fft_exec_dir(self.handle, in_ptr, out_ptr, d, _stream_handle(stream))
+        if rc:
+            raise L.GbfftError(rc, "fft_exec")
 
     def numel(self) -> int:
         """Complex elements one execution reads and writes."""
@@ -125,8 +138,8 @@ class Plan:
         want = torch.complex128 if self.prec == L.FFT_PREC_FP64 else torch.complex64
         if x.dtype != want or not x.is_cuda or x.device != self.device:
             raise TypeError(f"expected a {want} tensor on {self.device}")
-        if x.numel() != self.numel():
-            raise ValueError(f"expected {self.numel()} elements, got {x.numel()}")
+        if x.numel() != self.points:
+            raise ValueError(f"expected {self.points} elements, got {x.numel()}")
         x = x.contiguous()
         if out is None:
             out = torch.empty_like(x)
@@ -139,8 +152,7 @@ class Plan:
     def exec_filter_ptr(self, in_ptr: int, out_ptr: int, filt_ptr: int, stream=None, dir: int = FORWARD) -> None:
         """Range compression IFFT(H * FFT(row)) of every row, or with
         dir=ADJOINT its adjoint IFFT(conj(H) * FFT(row)) (fft_exec_filter_dir)."""
-        rc = self.lib.fft_exec_filter_dir(self.handle, ctypes.c_void_p(in_ptr), ctypes.c_void_p(out_ptr),
-                                          ctypes.c_void_p(filt_ptr), int(dir), ctypes.c_void_p(_stream_handle(stream)))
+        rc = self.lib.fft_exec_filter_dir(self.handle, in_ptr, out_ptr, filt_ptr, int(dir), _stream_handle(stream))
         L.check(rc, "fft_exec_filter_dir")
 
     def status(self, stream=None) -> int:
@@ -202,17 +214,31 @@ def _check_input(x: torch.Tensor, min_dims: int = 1, allow_fp64: bool = False) -
         raise ValueError(f"expected at least {min_dims} dimension(s)")
 
 
+def _plan_1d(x, prec):
+    """The plan of x's rows, or None if there are none."""
+    n = x.shape[-1]
+    if x.numel() == 0 and n > 0:   # no rows: nothing to transform
+        return None
+    return get_plan("1d", (n,), x.numel() // n if n else 0, prec, x.device)
+
+
+def _plan_2d(x, prec):
+    ny, nx = x.shape[-2], x.shape[-1]
+    if x.numel() == 0 and ny * nx > 0:
+        return None
+    return get_plan("2d", (ny, nx), x.numel() // (ny * nx) if ny * nx else 0, prec, x.device)
+
+
+def _run(plan, x, dir):
+    return torch.empty_like(x) if plan is None else plan(x, dir=dir)
+
+
 class _FFT1d(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, dir, prec):
-        n = x.shape[-1]
         ctx.dir = dir
-        ctx.plan = None
-        if x.numel() == 0 and n > 0:   # no rows: nothing to transform
-            return torch.empty_like(x)
-        plan = get_plan("1d", (n,), x.numel() // n if n else 0, prec, x.device)
-        ctx.plan = plan
-        return plan(x, dir=dir)
+        ctx.plan = _plan_1d(x, prec)
+        return _run(ctx.plan, x, dir)
 
     @staticmethod
     def backward(ctx, g):
@@ -224,14 +250,9 @@ class _FFT1d(torch.autograd.Function):
 class _FFT2d(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, dir, prec):
-        ny, nx = x.shape[-2], x.shape[-1]
         ctx.dir = dir
-        ctx.plan = None
-        if x.numel() == 0 and ny * nx > 0:
-            return torch.empty_like(x)
-        plan = get_plan("2d", (ny, nx), x.numel() // (ny * nx) if ny * nx else 0, prec, x.device)
-        ctx.plan = plan
-        return plan(x, dir=dir)
+        ctx.plan = _plan_2d(x, prec)
+        return _run(ctx.plan, x, dir)
 
     @staticmethod
     def backward(ctx, g):
@@ -261,34 +282,46 @@ def _prec_for(x: torch.Tensor, prec):
     return "fp32" if prec is None else prec
 
 
+def _apply_1d(x, dir, prec):
+    _check_input(x, allow_fp64=True)
+    prec = _prec_for(x, prec)
+    if _direct(x):
+        return _run(_plan_1d(x, prec), x, dir)
+    return _FFT1d.apply(x, dir, prec)
+
+
+def _apply_2d(x, dir, prec):
+    _check_input(x, 2, allow_fp64=True)
+    prec = _prec_for(x, prec)
+    if _direct(x):
+        return _run(_plan_2d(x, prec), x, dir)
+    return _FFT2d.apply(x, dir, prec)
+
+
 def fft(x: torch.Tensor, prec=None) -> torch.Tensor:
     """Eq. 1 over the last dimension.  complex64 runs in FP32 (or a
     tensor-core precision): powers of two 2..2^28 and products 2^a 3^b 5^c 7^d
     up to 14336^2 (two passes above 14336).  complex128 runs in FP64: the same
     7-smooth lengths up to 7168^2 (powers of two up to 2^24; two passes above
     7168)."""
-    _check_input(x, allow_fp64=True)
-    return _FFT1d.apply(x, FORWARD, _prec_for(x, prec))
+    return _apply_1d(x, FORWARD, prec)
 
 
 def ifft(x: torch.Tensor, prec=None) -> torch.Tensor:
     """Eq. 2 over the last dimension (same lengths and precisions as fft)."""
-    _check_input(x, allow_fp64=True)
-    return _FFT1d.apply(x, INVERSE, _prec_for(x, prec))
+    return _apply_1d(x, INVERSE, prec)
 
 
 def fft2(x: torch.Tensor, prec=None) -> torch.Tensor:
     """2-D transform over the last two dimensions (rows, then columns).
     complex64: power-of-two sides up to 2^14 (any precision), or 7-smooth
     sides up to 14336 in FP32; complex128: 7-smooth sides up to 7168 in FP64."""
-    _check_input(x, 2, allow_fp64=True)
-    return _FFT2d.apply(x, FORWARD, _prec_for(x, prec))
+    return _apply_2d(x, FORWARD, prec)
 
 
 def ifft2(x: torch.Tensor, prec=None) -> torch.Tensor:
     """Eq. 2 in two dimensions (same sides and precisions as fft2)."""
-    _check_input(x, 2, allow_fp64=True)
-    return _FFT2d.apply(x, INVERSE, _prec_for(x, prec))
+    return _apply_2d(x, INVERSE, prec)
 
 
 def fft_many(packed: torch.Tensor, lengths, inverse: bool = False, prec="fp32", tuned: bool = False) -> torch.Tensor:
@@ -343,6 +376,8 @@ def range_compress(x: torch.Tensor, H: torch.Tensor) -> torch.Tensor:
         raise TypeError("H must be a complex64 CUDA tensor of shape (n,)")
     if H.device != x.device:
         raise ValueError("x and H must be on the same device")
+    if _direct(x):
+        return _run_filter(x.contiguous(), H.detach().contiguous())
     return _RangeCompress.apply(x.contiguous(), H.detach().contiguous())
 
 
@@ -405,6 +440,8 @@ def rfft(x: torch.Tensor) -> torch.Tensor:
     a 7-smooth FP64 length) -> complex128.  Differentiable."""
     if not isinstance(x, torch.Tensor) or x.dtype not in (torch.float32, torch.float64) or not x.is_cuda:
         raise TypeError("expected a float32 or float64 CUDA tensor")
+    if _direct(x):
+        return _run_real(x.contiguous(), x.shape[-1], FORWARD)
     return _RFFT.apply(x.contiguous())
 
 
@@ -418,6 +455,8 @@ def irfft(X: torch.Tensor, n: int | None = None) -> torch.Tensor:
         n = 2 * (X.shape[-1] - 1)
     if X.shape[-1] != n // 2 + 1:
         raise ValueError(f"irfft: {X.shape[-1]} values for length {n}")
+    if _direct(X):
+        return _run_real(X.contiguous(), int(n), INVERSE)
     return _IRFFT.apply(X.contiguous(), int(n))
 
 
