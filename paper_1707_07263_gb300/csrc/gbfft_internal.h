@@ -212,6 +212,7 @@ struct fft_plan {
   const gbfft::TileKernelInfo* kpfs;  // its variant staging the next transform by a bulk copy (or NULL;
                                       // kpf is then the fallback for inputs not 16-byte aligned)
   long long pf_grid;                  // its resident-CTA grid
+  void* d_tw32;                       // stage table of the row kernels with 32 points a thread (2^13, 2^14)
   const gbfft::TileKernelInfo* kradix;  // single pass with radix-8 / radix-4 passes (config radix), or NULL
   void* d_radtw;                        // its stage table (schedule of largest radix 2^radix_lgm)
   int radix_lgm;

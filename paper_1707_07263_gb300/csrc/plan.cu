@@ -187,6 +187,7 @@ static void free_plan(fft_plan* p) {
   if (p->d_tc) cudaFree(p->d_tc);
   if (p->d_rctw) cudaFree(p->d_rctw);
   if (p->d_radtw) cudaFree(p->d_radtw);
+  if (p->d_tw32) cudaFree(p->d_tw32);
   if (p->d_tables) cudaFree(p->d_tables);
   delete p;
 }
@@ -228,6 +229,20 @@ static void set_out_xf(TileArgs& a, const DirXf& x) {
   a.scale_out = (x.conj || x.scale != 1.0f) ? 1 : 0;
   a.sx = x.scale;
   a.sy = x.conj ? -x.scale : x.scale;
+}
+
+// The stage table of kernel k where its largest radix is 32, once per plan
+// (p->d_tw32; every such kernel of a plan has the plan's row length).
+static int build_row_table(fft_plan* p, const TileKernelInfo* k) {
+  if (k->lgm != 5 || p->d_tw32) return FFT_OK;
+  if (cudaMalloc(&p->d_tw32, (size_t)stage_tw_size(k->lg, false, 5) * 8 + 8) != cudaSuccess) return FFT_ERR_ALLOC;
+  if (launch_gen_stage_twiddles((float2*)p->d_tw32, k->lg, 0, false, 5) != cudaSuccess ||
+      cudaStreamSynchronize(0) != cudaSuccess)
+    return FFT_ERR_CUDA;
+  return FFT_OK;
+}
+static const float2* stage_table(const fft_plan* p, const TileKernelInfo* k, const float2* radix16) {
+  return k->lgm == 5 ? (const float2*)p->d_tw32 : radix16;
 }
 
 // ---- single on-chip pass -------------------------------------------------
@@ -289,6 +304,7 @@ static int exec_single(fft_plan* p, const float2* in, float2* out, int dir, cuda
     long long ntiles = a.tiles_per_batch;
     const long long grid = p->pf_grid < ntiles ? p->pf_grid : ntiles;
     int* st = p->d_status;
+    a.tw = stage_table(p, p->kpfs, a.tw);
     void* args[] = {(void*)&a, (void*)&ntiles, (void*)&st};
     return cudaLaunchKernel(p->kpfs->fn, dim3((unsigned)grid), dim3(p->kpfs->threads), args,
                             (size_t)p->kpfs->smem_bytes, s) == cudaSuccess
@@ -370,6 +386,7 @@ static int exec_passes(fft_plan* p, const float2* in, float2* out, int dir, cuda
       long long ntiles = d.ntiles;
       const long long grid = d.pf_grid < ntiles ? d.pf_grid : ntiles;
       int* st = p->d_status;
+      a.tw = stage_table(p, d.kpfs, a.tw);
       void* args[] = {(void*)&a, (void*)&ntiles, (void*)&st};
       rc = cudaLaunchKernel(d.kpfs->fn, dim3((unsigned)grid), dim3(d.kpfs->threads), args,
                             (size_t)d.kpfs->smem_bytes, s) == cudaSuccess
@@ -410,7 +427,8 @@ static int exec_filter_plan(fft_plan* p, const float2* in, float2* out, const fl
     a.in_sc = a.out_sc = L;
     a.in_sn = a.out_sn = 1;
     a.ncols = p->batch;
-    a.tw_rev = p->d_rctw ? (const float2*)p->d_rctw : p->tw1;
+    a.tw = stage_table(p, p->krc, p->tw1);
+    a.tw_rev = p->d_rctw ? (const float2*)p->d_rctw : a.tw;
     a.filt = filt;
     a.filt_mask = L - 1;
     a.filt_conj = conj_filt;
@@ -507,7 +525,7 @@ static int exec_real(fft_plan* p, const float2* in, float2* out, int dir, cudaSt
     base_args(a);
     a.in = in;
     a.out = out;
-    a.tw = p->tw1;
+    a.tw = stage_table(p, k, p->tw1);
     a.tiles_per_batch = (p->batch + C - 1) / C;
     a.ncols = p->batch;
     a.r_w = p->r_lo;   // one-level table W_N^k, k < M
@@ -692,6 +710,7 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
     if (p->prec == FFT_PREC_FP32) {
       p->krc = tile_kernel_rc(lgN);
       rc = prepare_kernel(p->krc);
+      if (!rc) rc = build_row_table(p, p->krc);
       if (rc) return rc;
       if (rc_persistent(lgN)) {
         int per_sm = 0, sms = 0, dev = 0;
@@ -703,10 +722,11 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
           return FFT_ERR_CUDA;
         p->rc_grid = (long long)per_sm * sms;
       }
-      if (lgN % 4 != 0 && lgN > 4) {
+      const int lgm = p->krc->lgm;
+      if (lgN % lgm != 0 && lgN > lgm) {
         // the fused kernel's second transform runs the remainder pass last
-        if (cudaMalloc(&p->d_rctw, (size_t)stage_tw_size(lgN, true) * 8) != cudaSuccess) return FFT_ERR_ALLOC;
-        if (launch_gen_stage_twiddles((float2*)p->d_rctw, lgN, 0, true) != cudaSuccess ||
+        if (cudaMalloc(&p->d_rctw, (size_t)stage_tw_size(lgN, true, lgm) * 8) != cudaSuccess) return FFT_ERR_ALLOC;
+        if (launch_gen_stage_twiddles((float2*)p->d_rctw, lgN, 0, true, lgm) != cudaSuccess ||
             cudaStreamSynchronize(0) != cudaSuccess)
           return FFT_ERR_CUDA;
       }
@@ -773,12 +793,14 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
       if (cfg->tma == 3 || (cfg->tma < 0 && (env_pf < 0 || env_pf == 3))) {
         p->kpfs = tile_kernel_pfs(lgN);
         rc = prepare_kernel(p->kpfs);
+        if (!rc) rc = build_row_table(p, p->kpfs);
         if (rc) return rc;
       }
       int per_sm = 0, sms = 0, dev = 0;
       cudaGetDevice(&dev);
       if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, p->kpfs ? p->kpfs->fn : p->kpf->fn, p->kpf->threads,
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, p->kpfs ? p->kpfs->fn : p->kpf->fn,
+                                                        p->kpfs ? p->kpfs->threads : p->kpf->threads,
                                                         (size_t)(p->kpfs ? p->kpfs->smem_bytes : p->kpf->smem_bytes)) !=
               cudaSuccess ||
           per_sm < 1)
@@ -1106,6 +1128,8 @@ static int build_2d(fft_plan* p, int ly, int lx) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kp->fn, kp->threads, (size_t)kp->smem_bytes) ==
             cudaSuccess &&
         per_sm >= 1) {
+      rc = build_row_table(p, kp);
+      if (rc) return rc;
       R.kpfs = kp;
       R.pf_grid = (long long)per_sm * sms;
     }
@@ -1366,6 +1390,7 @@ static int plan_real(fft_plan* p, int lgN) {
     if (!p->kr2c || !p->kc2r) return FFT_ERR_UNSUPPORTED;
     int rc = prepare_kernel(p->kr2c);
     if (!rc) rc = prepare_kernel(p->kc2r);
+    if (!rc) rc = build_row_table(p, p->kr2c);
     if (rc) return rc;
     p->k1 = p->kr2c;
     p->c1 = p->kr2c->C;

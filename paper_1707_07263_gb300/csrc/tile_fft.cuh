@@ -39,6 +39,7 @@
 #include "../../include/gbfft.h"
 #include "ct_trig.h"
 #include "fft_common.cuh"
+#include "fft_radix32.cuh"
 #include "tma_util.cuh"
 
 namespace gbfft {
@@ -104,8 +105,9 @@ __host__ __device__ constexpr int tc_row_pad(int C, bool in_cf, bool out_cf) {
 }
 
 // LGM: log2 of the largest radix, which is also the number of points each
-// thread holds (4: radix 16, every kernel but the autotuner's smaller-radix
-// single-pass variants, 3: radix 8, 2: radix 4).
+// thread holds (4: radix 16; 5: radix 32, the row kernels of 2^13 and 2^14,
+// row_lgm in tile_registry.h; 3 and 2: radix 8 and 4, the autotuner's
+// smaller-radix single-pass variants).
 template <int LG, int C, bool IN_CF, bool OUT_CF, int IDX = 0, int LGM = 4>
 struct TileCfg {
   static constexpr int L = 1 << LG;
@@ -237,6 +239,7 @@ __device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, 
     if constexpr (R >= 4) w[2] = __ldg(t + NS + k);
     if constexpr (R >= 8) w[4] = __ldg(t + 2 * NS + k);
     if constexpr (R >= 16) w[8] = __ldg(t + 3 * NS + k);
+    if constexpr (R >= 32) w[16] = __ldg(t + 4 * NS + k);
     if constexpr (R >= 4) w[3] = cmul(w[1], w[2]);
     if constexpr (R >= 8) {
       w[5] = cmul(w[4], w[1]);
@@ -246,6 +249,10 @@ __device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, 
     if constexpr (R >= 16) {
 #pragma unroll
       for (int r = 1; r < 8; ++r) w[8 + r] = cmul(w[8], w[r]);
+    }
+    if constexpr (R >= 32) {
+#pragma unroll
+      for (int r = 1; r < 16; ++r) w[16 + r] = cmul(w[16], w[r]);
     }
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r]);
@@ -311,7 +318,7 @@ __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_
 
   // ---- gather the R inputs of each butterfly ----
   if constexpr (FIRST && PRE == 4) {
-    static_assert(NB == 1 && (R == 16 || R == L), "register hand-over needs a one-butterfly first pass");
+    static_assert(NB == 1 && (R == (1 << LGM) || R == L), "register hand-over needs a one-butterfly first pass");
   } else if constexpr (FIRST) {
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
@@ -716,14 +723,14 @@ __global__ void __launch_bounds__(TileCfg<LG, 1, false, false>::T)
 // The wait on the barrier is bounded: on expiry the CTA records
 // FFT_ERR_TIMEOUT in `status`, waits once more (bounded) for the copy in
 // flight, and returns.
-template <int LG>
-constexpr int pfs_smem_bytes() { return TileCfg<LG, 1, false, false>::SMEM_BYTES + 16; }
+template <int LG, int LGM = 4>
+constexpr int pfs_smem_bytes() { return TileCfg<LG, 1, false, false, 0, LGM>::SMEM_BYTES + 16; }
 
-template <int LG>
-__global__ void __launch_bounds__(TileCfg<LG, 1, false, false>::T)
+template <int LG, int LGM = 4>
+__global__ void __launch_bounds__(TileCfg<LG, 1, false, false, 0, LGM>::T, LGM == 5 && LG <= 13 ? 2 : 0)
     tile_fft_pfs_kernel(const TileArgs a, long long ntiles, int* status) {
   extern __shared__ float2 smem[];
-  using Cfg = TileCfg<LG, 1, false, false>;
+  using Cfg = TileCfg<LG, 1, false, false, 0, LGM>;
   static_assert(Cfg::NST > 1 && Cfg::SM_TILE >= Cfg::L, "the staged copy must fit the exchange buffer");
   constexpr int BYTES = Cfg::L * 8;
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + Cfg::SM_TILE);
@@ -753,7 +760,7 @@ __global__ void __launch_bounds__(TileCfg<LG, 1, false, false>::T)
     parity ^= 1;
     // (no closing barrier: the next transform starts with the wait on its copy,
     // which the last pass issued after every thread had read the buffer)
-    tile_stage<LG, 1, false, false, 0, false, 6, 4>(v, smem, a, next, a.out + t * a.out_gstride, t, 0, nullptr);
+    tile_stage<LG, 1, false, false, 0, false, 6, 4, false, LGM>(v, smem, a, next, a.out + t * a.out_gstride, t, 0, nullptr);
   }
 }
 
@@ -761,7 +768,10 @@ __global__ void __launch_bounds__(TileCfg<LG, 1, false, false>::T)
 // thread at every size (measured on GB300: more registers than the default
 // heuristic picks speed up 2^13 and 2^14; 48 at 256 threads spills and
 // does not help 2^12).
-__host__ __device__ constexpr int rc_min_blocks(int threads) { return threads <= 256 ? 4 : (threads <= 512 ? 2 : 1); }
+__host__ __device__ constexpr int rc_min_blocks(int threads, int lgm = 4) {
+  const int b = threads <= 256 ? 4 : (threads <= 512 ? 2 : 1);
+  return lgm == 5 ? b / 2 : b;   // 128 registers: 32 points a thread
+}
 
 // Range compression of C contiguous rows per CTA (fast convolution, the
 // FFT-based SAR step of Sec. 3 and Sec. 4): y = IDFT(H * DFT(x)) with one
@@ -774,11 +784,12 @@ __host__ __device__ constexpr int rc_min_blocks(int threads) { return threads <=
 // next row into L2 (as tile_fft_pf_kernel); shorter rows take one tile per CTA.
 __host__ __device__ constexpr bool rc_persistent(int lg) { return lg == 14; }
 
-template <int LG, int C>
-__global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T, rc_min_blocks(TileCfg<LG, C, false, false>::T))
+template <int LG, int C, int LGM = 4>
+__global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
+                                  rc_min_blocks(TileCfg<LG, C, false, false, 0, LGM>::T, LGM))
     tile_rc_kernel(const TileArgs a, long long ntiles) {
   extern __shared__ float2 smem[];
-  using Cfg = TileCfg<LG, C, false, false>;
+  using Cfg = TileCfg<LG, C, false, false, 0, LGM>;
   float2 v[Cfg::P];
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
     if constexpr (rc_persistent(LG)) {
@@ -794,7 +805,7 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T, rc_min_blocks
       const long long b = t / a.tiles_per_batch;
       const long long g = t - b * a.tiles_per_batch;
       const float2* gin = a.in + b * a.in_bstride + g * a.in_gstride;
-      tile_stage<LG, C, false, false, 0, false, 0, 2>(v, smem, a, gin, nullptr, g * C, b, nullptr);
+      tile_stage<LG, C, false, false, 0, false, 0, 2, false, LGM>(v, smem, a, gin, nullptr, g * C, b, nullptr);
     }
     {
       // The tile index is passed through an opaque move, so that the output
@@ -805,7 +816,7 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T, rc_min_blocks
       const long long b = tt / a.tiles_per_batch;
       const long long g = tt - b * a.tiles_per_batch;
       float2* gout = a.out + b * a.out_bstride + g * a.out_gstride;
-      tile_stage<LG, C, false, false, 0, false, 4, 0, true>(v, smem, a, nullptr, gout, g * C, b, nullptr);
+      tile_stage<LG, C, false, false, 0, false, 4, 0, true, LGM>(v, smem, a, nullptr, gout, g * C, b, nullptr);
     }
     if constexpr (!rc_persistent(LG)) break;
     __syncthreads();   // the next tile's first exchange overwrites this one's
@@ -817,16 +828,19 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T, rc_min_blocks
 // z[m] = x[2m] + i x[2m+1] is transformed on chip (Z = Eq. 1 of length L) and
 // the last pass turns Z into X[0..L] (POST == 3), written to rows of L + 1
 // complex values (out_sc).  One read and one write of every value.
-template <int LG, int C>
-__global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T) tile_r2c_kernel(const TileArgs a) {
+template <int LG, int C, int LGM = 4>
+__global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
+                                  LGM == 5 ? rc_min_blocks(TileCfg<LG, C, false, false, 0, LGM>::T, LGM) : 0)
+    tile_r2c_kernel(const TileArgs a) {
   extern __shared__ float2 smem[];
-  using Cfg = TileCfg<LG, C, false, false>;
+  using Cfg = TileCfg<LG, C, false, false, 0, LGM>;
   const long long tile = blockIdx.x;
   const long long b = tile / a.tiles_per_batch;
   const long long g = tile - b * a.tiles_per_batch;
   float2 v[Cfg::P];
-  tile_stage<LG, C, false, false, 0, false, 0, 3>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
-                                                  a.out + b * a.out_bstride + g * a.out_gstride, g * C, b, nullptr);
+  tile_stage<LG, C, false, false, 0, false, 0, 3, false, LGM>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
+                                                              a.out + b * a.out_bstride + g * a.out_gstride, g * C, b,
+                                                              nullptr);
 }
 
 // Complex-to-real transform (the inverse of tile_r2c_kernel): rows of L + 1
@@ -834,17 +848,19 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T) tile_r2c_kern
 // Z[n] = E[n] + i O[n] from X[n] and X[L - n] (PRE == 5) and the tile runs
 // the inverse length-L transform by conjugation (conj_in = 1, a.sx = 1/L,
 // a.sy = -1/L); z[m] = x[2m] + i x[2m+1] is stored as L complex values.
-template <int LG, int C>
-__global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T, rc_min_blocks(TileCfg<LG, C, false, false>::T))
+template <int LG, int C, int LGM = 4>
+__global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
+                                  rc_min_blocks(TileCfg<LG, C, false, false, 0, LGM>::T, LGM))
     tile_c2r_kernel(const TileArgs a) {
   extern __shared__ float2 smem[];
-  using Cfg = TileCfg<LG, C, false, false>;
+  using Cfg = TileCfg<LG, C, false, false, 0, LGM>;
   const long long tile = blockIdx.x;
   const long long b = tile / a.tiles_per_batch;
   const long long g = tile - b * a.tiles_per_batch;
   float2 v[Cfg::P];
-  tile_stage<LG, C, false, false, 0, false, 5, 0>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
-                                                  a.out + b * a.out_bstride + g * a.out_gstride, g * C, b, nullptr);
+  tile_stage<LG, C, false, false, 0, false, 5, 0, false, LGM>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
+                                                              a.out + b * a.out_bstride + g * a.out_gstride, g * C, b,
+                                                              nullptr);
 }
 
 }  // namespace gbfft

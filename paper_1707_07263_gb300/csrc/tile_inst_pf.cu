@@ -16,11 +16,12 @@ const TileKernelInfo* tile_kernel_pf(int lg) {
   return &tab[lg - 12];
 }
 
-#define GBFFT_PFS(LG) \
-  {(const void*)&tile_fft_pfs_kernel<LG>, TileCfg<LG, 1, false, false>::T, pfs_smem_bytes<LG>(), LG, 1, MAP_JJ}
+#define GBFFT_PFS(LG, LGM) \
+  {(const void*)&tile_fft_pfs_kernel<LG, LGM>, TileCfg<LG, 1, false, false, 0, LGM>::T, pfs_smem_bytes<LG, LGM>(), LG, 1, \
+   MAP_JJ, LGM}
 
 const TileKernelInfo* tile_kernel_pfs(int lg) {
-  static const TileKernelInfo tab[] = {GBFFT_PFS(12), GBFFT_PFS(13), GBFFT_PFS(14)};
+  static const TileKernelInfo tab[] = {GBFFT_PFS(12, row_lgm(12)), GBFFT_PFS(13, row_lgm(13)), GBFFT_PFS(14, row_lgm(14))};
   if (lg < 12 || lg > 14) return nullptr;
   return &tab[lg - 12];
 }

@@ -6,8 +6,9 @@
 namespace gbfft {
 
 #define GBFFT_RC(LG)                                                                            \
-  {(const void*)&tile_rc_kernel<LG, jj_cols(LG)>, TileCfg<LG, jj_cols(LG), false, false>::T,    \
-   jj_cols(LG) * TileCfg<LG, jj_cols(LG), false, false>::LP * 8, LG, jj_cols(LG), MAP_JJ}
+  {(const void*)&tile_rc_kernel<LG, jj_cols(LG), row_lgm(LG)>,                                  \
+   TileCfg<LG, jj_cols(LG), false, false, 0, row_lgm(LG)>::T,                                   \
+   jj_cols(LG) * TileCfg<LG, jj_cols(LG), false, false, 0, row_lgm(LG)>::LP * 8, LG, jj_cols(LG), MAP_JJ, row_lgm(LG)}
 
 const TileKernelInfo* tile_kernel_rc(int lg) {
   static const TileKernelInfo tab[] = {
