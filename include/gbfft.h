@@ -104,7 +104,7 @@ enum {
  * on-chip pass per transform (Sec. 2.3.2: short data is not partitioned);
  * longer ones are split N = N1*N2 into a column pass with twiddle scaling and
  * a row pass through global memory (Sec. 2.3.2: two exchanges between shared
- * and global memory); from 2^22 the rows are split once more (three passes).
+ * and global memory); from 2^23 the rows are split once more (three passes).
  * Multi-pass plans need a workspace (fft_plan_workspace_bytes).
  * Builds the twiddle tables on the current device (FP64 sincospi rounded
  * once to FP32; Sec. 2.3.1 look-up table).  Returns NULL on error. */

@@ -169,6 +169,7 @@ int mixed_exec(fft_plan* p, const void* in, void* out, int conj, double sx, doub
 cudaError_t launch_gen_twiddles_n64(double2* tab, long long N, long long count, cudaStream_t s);
 
 cudaError_t launch_gen_stage_twiddles(float2* tab, int lg, cudaStream_t s, bool rev = false, int lgm = 4);
+cudaError_t launch_gen_stage_table(float2* tab, int lg, cudaStream_t s);
 cudaError_t launch_gen_power_twiddles(float2* tab, int lgN, long long count, long long step, cudaStream_t s);
 // Real-to-complex transforms of N = 2M reals, M a two-pass four-step length
 // with rows of 2^6..2^12 points: the even/odd split folded into the row pass
@@ -212,7 +213,6 @@ struct fft_plan {
   const gbfft::TileKernelInfo* kpfs;  // its variant staging the next transform by a bulk copy (or NULL;
                                       // kpf is then the fallback for inputs not 16-byte aligned)
   long long pf_grid;                  // its resident-CTA grid
-  void* d_tw32;                       // stage table of the row kernels with 32 points a thread (2^13, 2^14)
   const gbfft::TileKernelInfo* kradix;  // single pass with radix-8 / radix-4 passes (config radix), or NULL
   void* d_radtw;                        // its stage table (schedule of largest radix 2^radix_lgm)
   int radix_lgm;

@@ -129,8 +129,8 @@ static int noalloc_run(int64_t n, int64_t batch, int dir, const float2* in, floa
   float2* lo = tw2 + 4096;
   float2* hi = lo + 4096;
   const int s_lo = (lgN + 1) / 2;
-  if (launch_gen_stage_twiddles(tw1, lg1, s) != cudaSuccess) return FFT_ERR_CUDA;
-  if (launch_gen_stage_twiddles(tw2, lg2, s) != cudaSuccess) return FFT_ERR_CUDA;
+  if (launch_gen_stage_table(tw1, lg1, s) != cudaSuccess) return FFT_ERR_CUDA;
+  if (launch_gen_stage_table(tw2, lg2, s) != cudaSuccess) return FFT_ERR_CUDA;
   if (launch_gen_power_twiddles(lo, lgN, 1LL << s_lo, 1, s) != cudaSuccess) return FFT_ERR_CUDA;
   if (launch_gen_power_twiddles(hi, lgN, 1LL << (lgN - s_lo), 1LL << s_lo, s) != cudaSuccess) return FFT_ERR_CUDA;
 

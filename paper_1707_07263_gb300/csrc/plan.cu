@@ -9,7 +9,7 @@
 //               W_N^{n2*k1}, written to the workspace as Y[k1][n2];
 //       pass 2  row FFTs of length N2 of Y[k1][.], written transposed to
 //               X[k1 + N1*k2].
-//     From 2^22 the row length N2 is itself split once more (three passes,
+//     From 2^23 the row length N2 is itself split once more (three passes,
 //     N = N1*N2*N3), so that every pass's sub-FFT stays at most 2^12 points.
 //   * 2-D ny x nx: row FFTs, then column FFTs in place (Sec. 2.3.2: rows,
 //     then columns).
@@ -117,7 +117,7 @@ static int build_tables_multi(fft_plan* p, const int lgs[3], const int lgNs[2]) 
   int ss[2] = {0, 0};
   for (int i = 0; i < 3; ++i) {
     stage_off[i] = off;
-    off += align256((lgs[i] > 0 ? (size_t)stage_tw_size(lgs[i]) : 0) * 8 + 8);
+    off += align256((lgs[i] > 0 ? (size_t)stage_table_size(lgs[i]) : 0) * 8 + 8);
   }
   for (int i = 0; i < 2; ++i) {
     if (lgNs[i] > 0) {
@@ -149,7 +149,7 @@ static int build_tables_multi(fft_plan* p, const int lgs[3], const int lgNs[2]) 
   if (cudaMemsetAsync(p->d_status, 0, sizeof(int), s) != cudaSuccess) return FFT_ERR_CUDA;
   const float2* st[3] = {p->tw1, p->tw2, p->tw3};
   for (int i = 0; i < 3; ++i)
-    if (lgs[i] > 0 && launch_gen_stage_twiddles((float2*)st[i], lgs[i], s) != cudaSuccess) return FFT_ERR_CUDA;
+    if (lgs[i] > 0 && launch_gen_stage_table((float2*)st[i], lgs[i], s) != cudaSuccess) return FFT_ERR_CUDA;
   const float2* los[2] = {p->ft_lo, p->ft2_lo};
   const float2* his[2] = {p->ft_hi, p->ft2_hi};
   for (int i = 0; i < 2; ++i) {
@@ -187,7 +187,6 @@ static void free_plan(fft_plan* p) {
   if (p->d_tc) cudaFree(p->d_tc);
   if (p->d_rctw) cudaFree(p->d_rctw);
   if (p->d_radtw) cudaFree(p->d_radtw);
-  if (p->d_tw32) cudaFree(p->d_tw32);
   if (p->d_tables) cudaFree(p->d_tables);
   delete p;
 }
@@ -229,20 +228,6 @@ static void set_out_xf(TileArgs& a, const DirXf& x) {
   a.scale_out = (x.conj || x.scale != 1.0f) ? 1 : 0;
   a.sx = x.scale;
   a.sy = x.conj ? -x.scale : x.scale;
-}
-
-// The stage table of kernel k where its largest radix is 32, once per plan
-// (p->d_tw32; every such kernel of a plan has the plan's row length).
-static int build_row_table(fft_plan* p, const TileKernelInfo* k) {
-  if (k->lgm != 5 || p->d_tw32) return FFT_OK;
-  if (cudaMalloc(&p->d_tw32, (size_t)stage_tw_size(k->lg, false, 5) * 8 + 8) != cudaSuccess) return FFT_ERR_ALLOC;
-  if (launch_gen_stage_twiddles((float2*)p->d_tw32, k->lg, 0, false, 5) != cudaSuccess ||
-      cudaStreamSynchronize(0) != cudaSuccess)
-    return FFT_ERR_CUDA;
-  return FFT_OK;
-}
-static const float2* stage_table(const fft_plan* p, const TileKernelInfo* k, const float2* radix16) {
-  return k->lgm == 5 ? (const float2*)p->d_tw32 : radix16;
 }
 
 // ---- single on-chip pass -------------------------------------------------
@@ -304,7 +289,6 @@ static int exec_single(fft_plan* p, const float2* in, float2* out, int dir, cuda
     long long ntiles = a.tiles_per_batch;
     const long long grid = p->pf_grid < ntiles ? p->pf_grid : ntiles;
     int* st = p->d_status;
-    a.tw = stage_table(p, p->kpfs, a.tw);
     void* args[] = {(void*)&a, (void*)&ntiles, (void*)&st};
     return cudaLaunchKernel(p->kpfs->fn, dim3((unsigned)grid), dim3(p->kpfs->threads), args,
                             (size_t)p->kpfs->smem_bytes, s) == cudaSuccess
@@ -386,7 +370,6 @@ static int exec_passes(fft_plan* p, const float2* in, float2* out, int dir, cuda
       long long ntiles = d.ntiles;
       const long long grid = d.pf_grid < ntiles ? d.pf_grid : ntiles;
       int* st = p->d_status;
-      a.tw = stage_table(p, d.kpfs, a.tw);
       void* args[] = {(void*)&a, (void*)&ntiles, (void*)&st};
       rc = cudaLaunchKernel(d.kpfs->fn, dim3((unsigned)grid), dim3(d.kpfs->threads), args,
                             (size_t)d.kpfs->smem_bytes, s) == cudaSuccess
@@ -427,8 +410,7 @@ static int exec_filter_plan(fft_plan* p, const float2* in, float2* out, const fl
     a.in_sc = a.out_sc = L;
     a.in_sn = a.out_sn = 1;
     a.ncols = p->batch;
-    a.tw = stage_table(p, p->krc, p->tw1);
-    a.tw_rev = p->d_rctw ? (const float2*)p->d_rctw : a.tw;
+    a.tw_rev = p->d_rctw ? (const float2*)p->d_rctw : p->tw1;
     a.filt = filt;
     a.filt_mask = L - 1;
     a.filt_conj = conj_filt;
@@ -471,6 +453,8 @@ static int exec_filter_plan(fft_plan* p, const float2* in, float2* out, const fl
       }
       const int rc = (d.kcol && coltma_usable(d.kcol, a, a.in))
                          ? coltma_launch(d.kcol, a, d.ntiles, d.col_grid, p->d_status, s)
+                     : (d.kst && rowtmas_usable(d.kst, a, a.out, d.ntiles))   // not where the filter multiplies
+                         ? rowtmas_launch(d.kst, a, d.ntiles, s)
                          : launch_tile(d.k, a, d.ntiles, s);
       if (rc) return rc;
     }
@@ -525,7 +509,7 @@ static int exec_real(fft_plan* p, const float2* in, float2* out, int dir, cudaSt
     base_args(a);
     a.in = in;
     a.out = out;
-    a.tw = stage_table(p, k, p->tw1);
+    a.tw = p->tw1;
     a.tiles_per_batch = (p->batch + C - 1) / C;
     a.ncols = p->batch;
     a.r_w = p->r_lo;   // one-level table W_N^k, k < M
@@ -660,8 +644,8 @@ int exec_plan(fft_plan* p, const void* in, void* out, int dir, cudaStream_t s) {
 // (or tma < 0) take the defaults: one on-chip pass up to 2^14 (radix-8 passes
 // at 2^5 and 2^6, TMA-staged for 2^9..2^11, persistent with the next transform
 // staged into the exchange buffer at 2^13 and 2^14), two passes
-// below 2^22 (2^8-point column tiles from 2^16 to 2^20, else the even split),
-// three passes 2^8 * 2^8 * rest from 2^22; as many adjacent columns per CTA
+// below 2^23 (2^7 to 2^10-point column tiles), three passes 2^8 * 2^8 * rest
+// from 2^23; as many adjacent columns per CTA
 // as fit 2^13 points (at most 16).
 static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
   fft_plan_config dflt;
@@ -710,7 +694,6 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
     if (p->prec == FFT_PREC_FP32) {
       p->krc = tile_kernel_rc(lgN);
       rc = prepare_kernel(p->krc);
-      if (!rc) rc = build_row_table(p, p->krc);
       if (rc) return rc;
       if (rc_persistent(lgN)) {
         int per_sm = 0, sms = 0, dev = 0;
@@ -793,7 +776,6 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
       if (cfg->tma == 3 || (cfg->tma < 0 && (env_pf < 0 || env_pf == 3))) {
         p->kpfs = tile_kernel_pfs(lgN);
         rc = prepare_kernel(p->kpfs);
-        if (!rc) rc = build_row_table(p, p->kpfs);
         if (rc) return rc;
       }
       int per_sm = 0, sms = 0, dev = 0;
@@ -826,8 +808,10 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
     return build_tables(p, lgN, 0, 0);
   }
   p->kind = KIND_FOURSTEP;
-  // measured on GB300 (autotuner): three passes 2^8 * 2^8 * rest from 2^22 up
-  int npass = cfg->npass >= 2 ? cfg->npass : ((lgN >= 22) ? 3 : 2);
+  // measured on GB300 (autotuner, per 2^26 points): three passes 2^8 * 2^8 *
+  // rest from 2^23 up (518 us against 547); at 2^22 two, 2^10 * 2^12, since the
+  // staged 2^10-point columns (474 against 527)
+  int npass = cfg->npass >= 2 ? cfg->npass : ((lgN >= 23) ? 3 : 2);
   const int force_np = env_int("GBFFT_PASSES", 0);
   if (cfg->npass < 2 && (force_np == 2 || force_np == 3)) npass = force_np;
   if (npass == 3 && lgN < 3) return FFT_ERR_UNSUPPORTED;
@@ -840,8 +824,8 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
     // for 2^8 x 2^12); 2^8 x 2^8 at 2^16; beyond 2^20, the even split
     // (tensor-core plans keep the even split their kernels are compiled for)
     const bool fp32 = p->prec == FFT_PREC_FP32;
-    static const int kLg2Default[5] = {8, 10, 10, 11, 10};   // lgN = 16..20
-    int lg2 = (fp32 && lgN >= 16 && lgN <= 20) ? kLg2Default[lgN - 16] : (lgN + 1) / 2;
+    static const int kLg2Default[7] = {8, 10, 10, 11, 10, 11, 12};   // lgN = 16..22
+    int lg2 = (fp32 && lgN >= 16 && lgN <= 22) ? kLg2Default[lgN - 16] : (lgN + 1) / 2;
     const int force_lg1 = cfg->lg1 > 0 ? cfg->lg1 : env_int("GBFFT_FORCE_SPLIT", 0);
     if (force_lg1 > 0 && force_lg1 < lgN && lgN - force_lg1 <= 14 && force_lg1 <= 14) lg2 = lgN - force_lg1;
     const int lg1 = lgN - lg2;
@@ -910,7 +894,7 @@ static int plan_1d(fft_plan* p, int lgN, const fft_plan_config* cfg) {
   //   B  per k1, columns of length N2 over stride N3 of the M-point
   //      row, scaled by W_M^{n3*k2}                                   ws -> ws (in place)
   //   C  rows of length N3, written to X[k1 + N1*k2 + N1*N2*k3]      ws -> out
-  // measured on GB300: 2^8 x 2^8 x rest from 2^22 to 2^28 (rest <= 2^12)
+  // measured on GB300: 2^8 x 2^8 x rest to 2^28 (rest <= 2^12)
   int l1 = (lgN >= 22 && lgN <= 28) ? 8 : (lgN + 2) / 3;
   int l2 = (lgN >= 22 && lgN <= 28) ? 8 : (lgN - l1 + 1) / 2;
   if (cfg->lg1 > 0) {
@@ -1128,14 +1112,15 @@ static int build_2d(fft_plan* p, int ly, int lx) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kp->fn, kp->threads, (size_t)kp->smem_bytes) ==
             cudaSuccess &&
         per_sm >= 1) {
-      rc = build_row_table(p, kp);
-      if (rc) return rc;
       R.kpfs = kp;
       R.pf_grid = (long long)per_sm * sms;
     }
   }
   if (!two) {
-    const int C = (int)std::min<long long>(env_int("GBFFT_FORCE_C2", default_cols(ly)), nx);
+    // columns per tile, measured on GB300 per 2^26 points: 2^6 32 instead of 16
+    // (64 x 1024 369 -> 346 us), 2^9 8 instead of 16 (512 x 8192 420 -> 411), the
+    // others as many as make 2^13 points
+    const int C = (int)std::min<long long>(env_int("GBFFT_FORCE_C2", ly == 6 ? 32 : ly == 9 ? 8 : default_cols(ly)), nx);
     const TileKernelInfo* kc = tile_kernel(MAP_CC, ly, C);
     if (!kc) return FFT_ERR_UNSUPPORTED;
     rc = prepare_kernel(kc);
@@ -1163,18 +1148,27 @@ static int build_2d(fft_plan* p, int ly, int lx) {
     p->npass = 2;
     p->launches = 2;
     p->ws_bytes = 0;
-    return attach_coltma(p, false);
+    // 2^10 rows: the kernel that stages the next tile in its exchange buffer
+    // (1024 x 4096 400 -> 356 us, 1024 x 256 380 -> 342); shorter columns measured
+    // slower staged (128 x 8192 358 -> 374)
+    return attach_coltma(p, ly == 10);
   }
-  int ly1 = ly / 2;
+  // two column passes 2^7 x rest, 32 columns per tile (256-byte runs), staged
+  // by tensor TMA (up to 2^13 rows).  Measured on GB300 per 2^26 points against
+  // the even split on the register path, 32 and 16 columns: 8192^2 557 -> 541
+  // us, 2048 x 8192 595 -> 551, 4096 x 16384 597 -> 562, 4096 x 256 527 -> 504
+  // (of every split 2^4..2^9 with 8..64 columns).  Images of fewer than 128
+  // columns have too few tiles a row for it (4096 x 4 647 -> 760): the even split.
+  const bool wide = nx >= 128;
+  int ly1 = wide ? 7 : ly / 2;
   const int env_ly1 = env_int("GBFFT_2D_LY1", 0);
   if (env_ly1 >= 1 && env_ly1 < ly && ly - env_ly1 <= 14) ly1 = env_ly1;
   const int ly2 = ly - ly1;
   const long long Y1 = 1LL << ly1, Y2 = 1LL << ly2;
-  // first column pass: 32 columns per tile where compiled (8192^2, 2^6 x 2^7:
-  // 611 -> 586 us against 16; 64 columns 599, other splits 590..660)
   const int ca_default = tile_kernel(MAP_CC, ly1, 32) ? 32 : default_cols(ly1);
+  const int cb_default = wide && tile_kernel(MAP_CC, ly2, 32) ? 32 : default_cols(ly2);
   const int ca = (int)std::min<long long>(env_int("GBFFT_2D_CA", ca_default), nx);
-  const int cb = (int)std::min<long long>(env_int("GBFFT_2D_CB", default_cols(ly2)), nx);
+  const int cb = (int)std::min<long long>(env_int("GBFFT_2D_CB", cb_default), nx);
   const TileKernelInfo* ka = tile_kernel(MAP_CC, ly1, ca);
   const TileKernelInfo* kb = tile_kernel(MAP_CC, ly2, cb);
   if (!ka || !kb) return FFT_ERR_UNSUPPORTED;
@@ -1233,7 +1227,7 @@ static int build_2d(fft_plan* p, int ly, int lx) {
   p->npass = 3;
   p->launches = 3;
   p->ws_bytes = (size_t)img * (size_t)p->batch * 8;
-  return attach_coltma(p, false);
+  return attach_coltma(p, wide && ly <= 13);
 }
 
 }  // namespace gbfft
@@ -1390,7 +1384,6 @@ static int plan_real(fft_plan* p, int lgN) {
     if (!p->kr2c || !p->kc2r) return FFT_ERR_UNSUPPORTED;
     int rc = prepare_kernel(p->kr2c);
     if (!rc) rc = prepare_kernel(p->kc2r);
-    if (!rc) rc = build_row_table(p, p->kr2c);
     if (rc) return rc;
     p->k1 = p->kr2c;
     p->c1 = p->kr2c->C;

@@ -31,14 +31,15 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
                : "memory");
 }
 
-template <int LG, int C>
-__global__ void __launch_bounds__(TileCfg<LG, C, false, true>::T)
+template <int LG, int C, int LGM>
+__global__ void __launch_bounds__(TileCfg<LG, C, false, true, 0, LGM>::T,
+                                  LGM == 5 ? 512 / TileCfg<LG, C, false, true, 0, LGM>::T : 0)
     row_tmas_kernel(const __grid_constant__ CUtensorMap omap, const TileArgs a) {
   static_assert((1 << LG) >= 256 && (C % 2) == 0, "boxes of C x 256 elements, 16-byte rows");
   constexpr int L = 1 << LG;
   extern __shared__ __align__(128) float2 rt_smem[];
   const long long tile = blockIdx.x;
-  tile_body<LG, C, false, true, false, 0, 7>(a, tile, rt_smem);
+  tile_body<LG, C, false, true, false, 0, 7, LGM>(a, tile, rt_smem);
   // the dense [k][c] tile is complete (mode 7 ends with a barrier)
   if (threadIdx.x == 0) {
     const long long b = tile / a.tiles_per_batch;
@@ -53,8 +54,8 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, true>::T)
 }
 
 #define GBFFT_ROWTMAS(LG, C) \
-  {(const void*)&row_tmas_kernel<LG, C>, TileCfg<LG, C, false, true>::T, TileCfg<LG, C, false, true>::SMEM_BYTES, \
-   LG, C, MAP_JC}
+  {(const void*)&row_tmas_kernel<LG, C, LG == 10 ? 5 : 4>, TileCfg<LG, C, false, true, 0, LG == 10 ? 5 : 4>::T, \
+   TileCfg<LG, C, false, true, 0, LG == 10 ? 5 : 4>::SMEM_BYTES, LG, C, MAP_JC, LG == 10 ? 5 : 4}
 
 // Rows of 2^10 and 2^11 points, four per CTA (256 / 512 threads), and of
 // 2^10 with eight (512 threads), where the plain store path is queue-bound.

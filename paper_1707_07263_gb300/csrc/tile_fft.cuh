@@ -74,6 +74,13 @@ __host__ __device__ constexpr int stage_tw_size(int lg, bool rev = false, int lg
   return stage_tw_off(lg, radix_nst(lg, lgm), rev, lgm);
 }
 
+// The table of a length holds the radix-16 schedule and, where kernels with 32
+// points a thread are compiled (tile_registry.h), the radix-32 one after it.
+__host__ __device__ constexpr bool stage_has_32(int lg) { return lg == 10 || lg == 13 || lg == 14; }
+__host__ __device__ constexpr int stage_table_size(int lg) {
+  return stage_tw_size(lg) + (stage_has_32(lg) ? stage_tw_size(lg, false, 5) : 0);
+}
+
 __host__ __device__ constexpr int cmin(int a, int b) { return a < b ? a : b; }
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
@@ -118,7 +125,8 @@ struct TileCfg {
                                      : L + tc_row_pad<IDX>(C, IN_CF, OUT_CF);
   static constexpr int SM_TILE = NST > 1 ? C * LP : 0;   // complex entries
   static constexpr bool EPI = IN_CF && OUT_CF;            // column pass: may carry the four-step twiddle
-  static constexpr int SM_EPI = EPI ? C * 16 : 0;         // four-step per-column step table
+  static constexpr int EPI_Q = LGM == 5 ? 32 : 16;        // outputs of a last-pass butterfly (at most)
+  static constexpr int SM_EPI = EPI ? C * EPI_Q : 0;      // four-step per-column step table
   static constexpr int SMEM_BYTES = (SM_TILE + SM_EPI) * 8;
 };
 
@@ -259,10 +267,18 @@ __device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, 
   }
 }
 
+// Called by the last pass of a tile once every thread has read its inputs from
+// the exchange buffer (a persistent kernel starts the next tile's copy there).
+struct NoHook {
+  static constexpr bool on = false;
+  __device__ __forceinline__ void operator()() const {}
+};
+
 // One pass S of the tile: gather, twiddle, R-point DFT, scatter (with the
 // barriers that separate it from its neighbours).
 //   PRE  0: first pass reads global memory; 1: two-CTA radix-2 split;
-//        2: first pass reads a TMA-staged box; 4: the first pass's inputs are
+//        2: first pass reads a TMA-staged box [n][c] (9: one that lies in the
+//        exchange buffer itself); 4: the first pass's inputs are
 //        already in registers (left there by a POST == 2 transform), no conj_in;
 //        5: first pass builds Z[n] = E[n] + i O[n] of a complex-to-real
 //        transform from X[n] and X[L - n] of rows of L + 1 values (C2R);
@@ -289,10 +305,11 @@ __device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, 
 //        PRE == 4, REV transform (radix-16 first pass: thread j reads n = j +
 //        r*L/16) without an exchange; lengths below 16 are one pass either way.
 template <int LG, int C, bool IN_CF, bool OUT_CF, int S, bool OFFS = false, int PRE = 0, int IDX = 0,
-          int POST = 0, bool REV = false, int LGM = 4>
+          int POST = 0, bool REV = false, int LGM = 4, typename Hook = NoHook>
 __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_CF, 0, LGM>::P], float2* sm,
                                           const TileArgs& a, const float2* gin, float2* gout,
-                                          long long col0, long long bidx, const float2* epi_tab) {
+                                          long long col0, long long bidx, const float2* epi_tab,
+                                          const Hook& hook = Hook()) {
   using Cfg = TileCfg<LG, C, IN_CF, OUT_CF, IDX, LGM>;
   constexpr int L = Cfg::L, P = Cfg::P, T = Cfg::T, NST = Cfg::NST, LP = Cfg::LP;
   constexpr int LGR = radix_lgr(LG, S, REV, LGM), R = 1 << LGR;
@@ -381,7 +398,7 @@ __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_
           x2[0] = make_float2(x2[0].x * em, 0.f);
         }
         c2r_combine<R>(v + i * R, x1, x2, w0);
-      } else if constexpr (PRE == 2) {
+      } else if constexpr (PRE == 2 || PRE == 9) {
         // column tile already staged in shared memory by a tensor TMA copy,
         // laid out [n][c] (gin points at it)
 #pragma unroll
@@ -428,6 +445,10 @@ __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_
       }
     }
   }
+  if constexpr (LAST && !FIRST && Hook::on) {
+    __syncthreads();
+    hook();
+  }
   if constexpr (LAST && POST == 4 && !FIRST) {
     // every thread holds its last-pass inputs: the buffer now receives the
     // next tile's rows while this pass computes and stores
@@ -440,7 +461,8 @@ __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_
 
   // ---- twiddles W_{Ns*R}^{r*(j mod Ns)} ----
   if constexpr (NS > 1) {
-    const float2* t = (REV ? a.tw_rev : a.tw) + stage_tw_off(LG, S, REV, LGM);
+    static_assert(LGM != 5 || stage_has_32(LG), "no radix-32 table");
+    const float2* t = (REV ? a.tw_rev : a.tw + (LGM == 5 ? stage_tw_size(LG) : 0)) + stage_tw_off(LG, S, REV, LGM);
 #pragma unroll
     for (int i = 0; i < NB; ++i) apply_stage_twiddle<R>(v + i * R, t, NS, jj[i] & (NS - 1));
   }
@@ -594,7 +616,7 @@ __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_
   } else {
     // all reads of this pass (or, for PRE == 4, of the previous transform's
     // last pass) are done
-    if constexpr (!FIRST || PRE == 4 || PRE == 6) __syncthreads();
+    if constexpr (!FIRST || PRE == 4 || PRE == 6 || PRE == 9) __syncthreads();
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
       const int j = jj[i];
@@ -613,13 +635,30 @@ __device__ __forceinline__ void tile_pass(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_
 }
 
 template <int LG, int C, bool IN_CF, bool OUT_CF, int S, bool OFFS = false, int PRE = 0, int POST = 0,
-          bool REV = false, int LGM = 4>
+          bool REV = false, int LGM = 4, typename Hook = NoHook>
 __device__ __forceinline__ void tile_stage(float2 (&v)[TileCfg<LG, C, IN_CF, OUT_CF, 0, LGM>::P], float2* sm,
                                            const TileArgs& a, const float2* gin, float2* gout,
-                                           long long col0, long long bidx, const float2* epi_tab) {
-  tile_pass<LG, C, IN_CF, OUT_CF, S, OFFS, PRE, 0, POST, REV, LGM>(v, sm, a, gin, gout, col0, bidx, epi_tab);
+                                           long long col0, long long bidx, const float2* epi_tab,
+                                           const Hook& hook = Hook()) {
+  tile_pass<LG, C, IN_CF, OUT_CF, S, OFFS, PRE, 0, POST, REV, LGM, Hook>(v, sm, a, gin, gout, col0, bidx, epi_tab,
+                                                                         hook);
   if constexpr (S + 1 < TileCfg<LG, C, IN_CF, OUT_CF, 0, LGM>::NST)
-    tile_stage<LG, C, IN_CF, OUT_CF, S + 1, OFFS, PRE, POST, REV, LGM>(v, sm, a, gin, gout, col0, bidx, epi_tab);
+    tile_stage<LG, C, IN_CF, OUT_CF, S + 1, OFFS, PRE, POST, REV, LGM, Hook>(v, sm, a, gin, gout, col0, bidx, epi_tab,
+                                                                             hook);
+}
+
+// The per-column step factors W_N^{n2*NS_last*q} of a column tile, entry q*C + c.
+template <int LG, int C, int LGM>
+__device__ __forceinline__ void tile_step_table(const TileArgs& a, long long col0, long long b, float2* epi_tab) {
+  using Cfg = TileCfg<LG, C, true, true, 0, LGM>;
+  constexpr int NS_LAST = 1 << radix_lgns(LG, Cfg::NST - 1, false, LGM);
+  for (int e = threadIdx.x; e < C * Cfg::EPI_Q; e += Cfg::T) {
+    const int q = e / C, c = e - q * C;
+    const unsigned n2 = a.ft_by_batch ? (unsigned)b : (unsigned)(col0 + c);
+    const unsigned m = (n2 * (unsigned)NS_LAST * (unsigned)q) & ((1u << a.ft_lgN) - 1u);
+    const unsigned mask = (1u << a.ft_s) - 1u;
+    epi_tab[e] = cmul(__ldg(a.ft_lo + (m & mask)), __ldg(a.ft_hi + (m >> a.ft_s)));
+  }
 }
 
 // One tile of a pass: tile index `tile` of the launch described by `a`, using
@@ -642,18 +681,11 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, long long tile, flo
   const float2* gin = a.in + b2 * a.in_b2stride + b * a.in_bstride + g * a.in_gstride;
   float2* gout = a.out + b2 * a.out_b2stride + b * a.out_bstride + g * a.out_gstride;
 
-  if (Cfg::EPI && a.ft_lgN) {
-    // per-column step factors W_N^{n2*NS_last*q}, q = 0..15
-    constexpr int NS_LAST = 1 << radix_lgns(LG, Cfg::NST - 1, false, LGM);
-    for (int e = threadIdx.x; e < C * 16; e += Cfg::T) {
-      const int q = e / C, c = e - q * C;   // entry q*C + c
-      const unsigned n2 = a.ft_by_batch ? (unsigned)b : (unsigned)(col0 + c);
-      const unsigned m = n2 * (unsigned)NS_LAST * (unsigned)q;
-      const unsigned mm = m & ((1u << a.ft_lgN) - 1u);
-      const unsigned mask = (1u << a.ft_s) - 1u;
-      epi_tab[e] = cmul(__ldg(a.ft_lo + (mm & mask)), __ldg(a.ft_hi + (mm >> a.ft_s)));
+  if constexpr (Cfg::EPI) {
+    if (a.ft_lgN) {
+      tile_step_table<LG, C, LGM>(a, col0, b, epi_tab);
+      if constexpr (Cfg::NST == 1) __syncthreads();
     }
-    if constexpr (Cfg::NST == 1) __syncthreads();
   }
 
   float2 v[Cfg::P];
@@ -682,7 +714,8 @@ __global__ void __launch_bounds__(TileCfg<LG, 1, false, false>::T, (LG >= 13 ? 2
 // and as many points per thread (single-pass variants the autotuner may pick;
 // stage table built for that schedule).
 template <int LG, int C, bool IN_CF, bool OUT_CF, int LGM = 4>
-__global__ void __launch_bounds__(TileCfg<LG, C, IN_CF, OUT_CF, 0, LGM>::T)
+__global__ void __launch_bounds__(TileCfg<LG, C, IN_CF, OUT_CF, 0, LGM>::T,
+                                  LGM == 5 ? cmax(1, 512 / TileCfg<LG, C, IN_CF, OUT_CF, 0, LGM>::T) : 0)
     tile_fft_kernel(const TileArgs a) {
   extern __shared__ float2 smem[];
   tile_body<LG, C, IN_CF, OUT_CF, false, 0, 0, LGM>(a, (long long)blockIdx.x, smem);

@@ -20,9 +20,9 @@ const TileKernelInfo* tile_kernel_cc_b(int lg, int C) {
       GBFFT_TK(9, 32, true, true, MAP_CC),
       GBFFT_TK(10, 1, true, true, MAP_CC),
       GBFFT_TK(10, 2, true, true, MAP_CC),
-      GBFFT_TK(10, 4, true, true, MAP_CC),
-      GBFFT_TK(10, 8, true, true, MAP_CC),
-      GBFFT_TK(10, 16, true, true, MAP_CC),
+      GBFFT_TK32(10, 4, true, true, MAP_CC),
+      GBFFT_TK32(10, 8, true, true, MAP_CC),
+      GBFFT_TK32(10, 16, true, true, MAP_CC),
   };
   for (const TileKernelInfo& k : tab)
     if (k.lg == lg && k.C == C) return &k;

@@ -39,7 +39,8 @@ constexpr int row_lgm(int lg) { return lg >= 13 ? 5 : 4; }
 const TileKernelInfo* tile_kernel_tma(int lg);
 constexpr int tma_exchange_width(int lg) { return lg >= 13 ? 4 : 8; }
 
-// Persistent tensor-TMA column kernels (tile_fft_tma2d.cuh), lengths 2^6..2^8.
+// Persistent tensor-TMA column kernels (tile_fft_tma2d.cuh), lengths 2^6..2^8
+// (box beside the exchange tile) and 2^10 (box in the exchange tile).
 const TileKernelInfo* tile_kernel_coltma(int lg, int C);
 bool coltma_usable(const TileKernelInfo* k, const TileArgs& a, const void* in);
 int coltma_launch(const TileKernelInfo* k, const TileArgs& a, long long ntiles, int grid, int* status,
@@ -87,6 +88,15 @@ const TileKernelInfo* tile_kernel_cc_c(int lg, int C);
 const TileKernelInfo* tile_kernel_jc_a(int lg, int C);
 const TileKernelInfo* tile_kernel_jc_b(int lg, int C);
 
+// Column and row passes of 2^10 points with four or more per tile: radix 32
+// (two passes, one exchange, where radix 16 takes three and two).  Measured per
+// 2^26 points: 1024 x 1024 images 384 -> 350 us, 2^26 582 -> 561; 2^20's row
+// pass at a copy's rate.  (Fewer columns leave too few threads a CTA; the real
+// rows folded into a 2^10-point row pass, one CTA of 16 rows per SM, measured
+// slower: rfft of 2^18 259 -> 267.)
+#define GBFFT_TK32(LG, C, ICF, OCF, MAP)                                                               \
+  {(const void*)&tile_fft_kernel<LG, C, ICF, OCF, 5>, TileCfg<LG, C, ICF, OCF, 0, 5>::T,                \
+   TileCfg<LG, C, ICF, OCF, 0, 5>::SMEM_BYTES, LG, C, MAP, 5}
 #define GBFFT_TK(LG, C, ICF, OCF, MAP)                                                         \
   {(const void*)&tile_fft_kernel<LG, C, ICF, OCF>, TileCfg<LG, C, ICF, OCF>::T,                 \
    TileCfg<LG, C, ICF, OCF>::SMEM_BYTES, LG, C, MAP}

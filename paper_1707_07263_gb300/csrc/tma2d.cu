@@ -16,10 +16,15 @@ namespace gbfft {
 #define GBFFT_COLTMA(LG, C) \
   {(const void*)&col_tma_kernel<LG, C>, ColTmaCfg<LG, C>::T, ColTmaCfg<LG, C>::SMEM_BYTES, LG, C, MAP_CC}
 
+// Box and exchange tile in one buffer (col_stage_kernel).
+#define GBFFT_COLSTAGE(LG, C, LGM) \
+  {(const void*)&col_stage_kernel<LG, C, LGM>, ColStageCfg<LG, C, LGM>::T, ColStageCfg<LG, C, LGM>::SMEM_BYTES, LG, C, \
+   MAP_CC, LGM}
+
 const TileKernelInfo* tile_kernel_coltma(int lg, int C) {
   static const TileKernelInfo tab[] = {GBFFT_COLTMA(6, 16), GBFFT_COLTMA(6, 32), GBFFT_COLTMA(7, 8),
                                        GBFFT_COLTMA(7, 16), GBFFT_COLTMA(7, 32), GBFFT_COLTMA(8, 8),
-                                       GBFFT_COLTMA(8, 16), GBFFT_COLTMA(8, 32)};
+                                       GBFFT_COLTMA(8, 16), GBFFT_COLTMA(8, 32), GBFFT_COLSTAGE(10, 8, 5)};
   for (const TileKernelInfo& k : tab)
     if (k.lg == lg && k.C == C) return &k;
   return nullptr;
@@ -45,7 +50,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 bool coltma_usable(const TileKernelInfo* k, const TileArgs& a, const void* in) {
   if (!k || !encode_fn()) return false;
   if (((uintptr_t)in & 15) || (a.in_sn & 1) || (a.in_bstride & 1) || (a.in_b2stride & 1)) return false;
-  if (a.in_sc != 1 || a.in_gstride != k->C || (k->C & 1) || (1 << k->lg) > 256) return false;
+  if (a.in_sc != 1 || a.in_gstride != k->C || (k->C & 1)) return false;
   return true;
 }
 
@@ -62,7 +67,7 @@ int coltma_launch(const TileKernelInfo* k, const TileArgs& a, long long ntiles, 
   const cuuint64_t dims[4] = {(cuuint64_t)a.ncols, (cuuint64_t)(1 << k->lg), (cuuint64_t)nz, (cuuint64_t)nw};
   const cuuint64_t zs = (cuuint64_t)a.in_bstride * 8;
   const cuuint64_t strides[3] = {(cuuint64_t)a.in_sn * 8, zs, a.nb1 ? (cuuint64_t)a.in_b2stride * 8 : zs * nz};
-  const cuuint32_t box[4] = {(cuuint32_t)k->C, (cuuint32_t)(1 << k->lg), 1, 1};
+  const cuuint32_t box[4] = {(cuuint32_t)k->C, (cuuint32_t)(k->lg < 8 ? 1 << k->lg : 256), 1, 1};   // rows: at most 256
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   CUtensorMap map;
   if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, (void*)a.in, dims, strides, box, estr,

@@ -162,6 +162,13 @@ cudaError_t launch_gen_stage_twiddles(float2* tab, int lg, cudaStream_t s, bool 
   return cudaGetLastError();
 }
 
+// The whole table of a length (stage_table_size entries).
+cudaError_t launch_gen_stage_table(float2* tab, int lg, cudaStream_t s) {
+  const cudaError_t e = launch_gen_stage_twiddles(tab, lg, s);
+  if (e != cudaSuccess || !stage_has_32(lg)) return e;
+  return launch_gen_stage_twiddles(tab + stage_tw_size(lg), lg, s, false, 5);
+}
+
 cudaError_t launch_gen_power_twiddles(float2* tab, int lgN, long long count, long long step, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
   const int threads = 256;
