@@ -26,12 +26,12 @@
 // takes its tile through plain FP64 sums (fx_special_tile); results outside
 // FP64's normal range take scalbn's rounding to subnormal numbers, zero or
 // infinity.
-// Radix 16 with 16 points a thread (128 registers, 16 warps an SM): 312
-// instructions a point at 4096, issued 40 % of the time; radix 8 with 64
-// registers takes one pass more and measured 407 us against 305.
-// Measured per 2^24 points on GB300, against the FP64 kernel: 64 641 -> 216 us,
-// 1000 1463 -> 486, 4096 1348 -> 305, 7000 1880 -> 610; two passes: 65536
-// 1961 -> 515, 2^20 2485 -> 701.
+// Radix 16 with 16 points a thread (128 registers, 16 warps an SM) issues about
+// 40 % of the time at 4096 points, held by latency and instruction fetch; radix
+// 8 with 64 registers takes one pass more and measured 407 us against 305.
+// Measured per 2^24 points on GB300, against the FP64 kernel: 64 641 -> 203 us,
+// 1000 1463 -> 387, 4096 1348 -> 294, 7000 1880 -> 667; two passes: 65536
+// 1961 -> 483, 2^20 2485 -> 719.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -227,8 +227,10 @@ __device__ __forceinline__ double2 fx_factor(const int4* p) {
                       ((double)w.i.h * 4294967296.0 + (double)w.i.l) * s);
 }
 
-// points a thread holds in the first and the middle passes
-constexpr int kFxPoints = 18;
+// points a thread holds in the first and the middle passes: with 20, two
+// butterflies of radix 10 and four of radix 5 fit 128 registers (18 before: 1000
+// points 469 -> 387 us per 2^24, 4000 610 -> 497)
+constexpr int kFxPoints = 20;
 template <int R>
 struct FxK {
   static constexpr int value = kFxPoints / R > 0 ? kFxPoints / R : 1;

@@ -142,22 +142,21 @@ GBFFT_HD long long fx_from_bits(long long bits, int E, int F) {
 }
 
 // q 2^ex as FP64 bits, rounded to nearest, for |q| < 2^63 and an ex for which
-// every such result is normal or zero (fx_normal).
+// every such result is normal or zero (fx_normal).  The conversion is one of the
+// FP64 pipe's, idle otherwise: 2 a clock and SM, against a leading-zero count, two
+// 64-bit shifts and the rounding on the integer units, which bound these kernels
+// (4096 points, 2^24 in all: 311 -> 291 us).
 constexpr bool fx_normal(int ex) { return ex >= -1022 && ex <= 958; }
 GBFFT_HD long long fx_to_bits(long long q, int ex) {
-  const int s = (int)(q >> 63);
-  const unsigned long long u = (unsigned long long)((q ^ (long long)s) - (long long)s);
 #ifdef __CUDA_ARCH__
-  const int lz = __clzll((long long)u);
+  const unsigned long long d = (unsigned long long)__double_as_longlong(__ll2double_rn(q));
 #else
-  const int lz = u ? __builtin_clzll(u) : 64;
+  const double f = (double)q;
+  unsigned long long d;
+  memcpy(&d, &f, 8);
 #endif
-  // leading bit to bit 62; 53 bits after rounding, or 2^53 on a carry
-  const unsigned long long m = ((u << ((lz - 1) & 63)) + 0x200) >> 10;
-  // the leading bit adds one to the exponent field
-  const int top = (int)(m >> 32) + ((1085 + ex - lz) << 20);
-  const unsigned long long b = ((unsigned long long)((unsigned)top | ((unsigned)s & 0x80000000u)) << 32) | (unsigned)m;
-  return u == 0 ? 0 : (long long)b;
+  const unsigned hi = (unsigned)(d >> 32);
+  return (long long)((unsigned long long)(hi ? hi + ((unsigned)ex << 20) : 0u) << 32 | (unsigned)d);
 }
 
 // bits of headroom an R-point DFT needs: ceil(log2(R sqrt 2)) (R - 1 additions

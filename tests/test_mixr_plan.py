@@ -55,7 +55,7 @@ int check(const Family& f, long long most, bool held, int points, int points_big
 int main() {
   int plans = 0;
   const int a = check(family_f32(), 14336, false, 25, 32, 384, 512, 16, plans);
-  const int b = check(family_fx(), 7168, true, 18, 18, 256, 512, 8, plans);
+  const int b = check(family_fx(), 7168, true, 20, 20, 256, 512, 8, plans);
   if (a < 0 || b < 0) return 1;
   printf("%d %d %d\n", a, b, plans);
   return 0;
