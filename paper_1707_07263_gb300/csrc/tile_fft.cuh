@@ -239,15 +239,16 @@ __device__ __forceinline__ void c2r_combine(float2* v, const float2* x1, const f
   }
 }
 
+// (w16: entry of the factor W^{16 k}, radix 32)
 template <int R>
-__device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, int NS, int k) {
+__device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, int NS, int k, int w16) {
   if constexpr (R >= 2) {
     float2 w[R];
     w[1] = __ldg(t + k);
     if constexpr (R >= 4) w[2] = __ldg(t + NS + k);
     if constexpr (R >= 8) w[4] = __ldg(t + 2 * NS + k);
     if constexpr (R >= 16) w[8] = __ldg(t + 3 * NS + k);
-    if constexpr (R >= 32) w[16] = __ldg(t + 4 * NS + k);
+    if constexpr (R >= 32) w[16] = __ldg(t + w16);
     if constexpr (R >= 4) w[3] = cmul(w[1], w[2]);
     if constexpr (R >= 8) {
       w[5] = cmul(w[4], w[1]);
@@ -265,6 +266,11 @@ __device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, 
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r]);
   }
+}
+
+template <int R>
+__device__ __forceinline__ void apply_stage_twiddle(float2* v, const float2* t, int NS, int k) {
+  apply_stage_twiddle<R>(v, t, NS, k, 4 * NS + k);
 }
 
 // Called by the last pass of a tile once every thread has read its inputs from
@@ -861,19 +867,17 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
 // z[m] = x[2m] + i x[2m+1] is transformed on chip (Z = Eq. 1 of length L) and
 // the last pass turns Z into X[0..L] (POST == 3), written to rows of L + 1
 // complex values (out_sc).  One read and one write of every value.
-template <int LG, int C, int LGM = 4>
-__global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
-                                  LGM == 5 ? rc_min_blocks(TileCfg<LG, C, false, false, 0, LGM>::T, LGM) : 0)
-    tile_r2c_kernel(const TileArgs a) {
+// Rows up to 2^9 reals; pair_r2c_kernel (real_pair.cuh) takes longer ones.
+template <int LG, int C>
+__global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T) tile_r2c_kernel(const TileArgs a) {
   extern __shared__ float2 smem[];
-  using Cfg = TileCfg<LG, C, false, false, 0, LGM>;
+  using Cfg = TileCfg<LG, C, false, false>;
   const long long tile = blockIdx.x;
   const long long b = tile / a.tiles_per_batch;
   const long long g = tile - b * a.tiles_per_batch;
   float2 v[Cfg::P];
-  tile_stage<LG, C, false, false, 0, false, 0, 3, false, LGM>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
-                                                              a.out + b * a.out_bstride + g * a.out_gstride, g * C, b,
-                                                              nullptr);
+  tile_stage<LG, C, false, false, 0, false, 0, 3>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
+                                                  a.out + b * a.out_bstride + g * a.out_gstride, g * C, b, nullptr);
 }
 
 // Complex-to-real transform (the inverse of tile_r2c_kernel): rows of L + 1
@@ -881,19 +885,18 @@ __global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
 // Z[n] = E[n] + i O[n] from X[n] and X[L - n] (PRE == 5) and the tile runs
 // the inverse length-L transform by conjugation (conj_in = 1, a.sx = 1/L,
 // a.sy = -1/L); z[m] = x[2m] + i x[2m+1] is stored as L complex values.
-template <int LG, int C, int LGM = 4>
-__global__ void __launch_bounds__(TileCfg<LG, C, false, false, 0, LGM>::T,
-                                  rc_min_blocks(TileCfg<LG, C, false, false, 0, LGM>::T, LGM))
+// Rows up to 2^5 reals; pair_c2r_kernel (real_pair.cuh) takes longer ones.
+template <int LG, int C>
+__global__ void __launch_bounds__(TileCfg<LG, C, false, false>::T, rc_min_blocks(TileCfg<LG, C, false, false>::T))
     tile_c2r_kernel(const TileArgs a) {
   extern __shared__ float2 smem[];
-  using Cfg = TileCfg<LG, C, false, false, 0, LGM>;
+  using Cfg = TileCfg<LG, C, false, false>;
   const long long tile = blockIdx.x;
   const long long b = tile / a.tiles_per_batch;
   const long long g = tile - b * a.tiles_per_batch;
   float2 v[Cfg::P];
-  tile_stage<LG, C, false, false, 0, false, 5, 0, false, LGM>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
-                                                              a.out + b * a.out_bstride + g * a.out_gstride, g * C, b,
-                                                              nullptr);
+  tile_stage<LG, C, false, false, 0, false, 5, 0>(v, smem, a, a.in + b * a.in_bstride + g * a.in_gstride,
+                                                  a.out + b * a.out_bstride + g * a.out_gstride, g * C, b, nullptr);
 }
 
 }  // namespace gbfft

@@ -23,15 +23,14 @@ struct TileKernelInfo {
 // Columns per CTA the JJ variant is compiled with for length 2^lg.
 constexpr int jj_cols(int lg) { return lg >= 12 ? 1 : (lg >= 4 ? (4096 >> lg) : 256); }
 
-// Largest radix (log2) of the staged persistent, range-compression and
-// real-data kernels: radix 32 with 32 points a thread (128 registers) at 2^13
-// and 2^14, radix 16 below.  At 2^13 and 2^14 a tile fills half an SM or all
-// of it and its warps meet at every exchange; 8 32 32 and 16 32 32 take two
-// exchanges where 2 16 16 16 and 4 16 16 16 take three, for about as many
-// instructions.  Measured per 2^26 points, radix 16 -> 32: 2^13 229 -> 202 us,
-// 2^14 243 -> 212 (a copy takes 158); range compression 355 -> 324 and 414 -> 373; real rows of 2^14 144 ->
-// 128 (forward), 151 -> 145 (inverse), of 2^15 180 -> 158 and 180 -> 172.  At
-// 2^12 three radix-16 passes already take two exchanges (170 us).
+// Largest radix (log2) of the staged persistent and range-compression kernels:
+// radix 32 with 32 points a thread (128 registers) at 2^13 and 2^14, radix 16
+// below.  At 2^13 and 2^14 a tile fills half an SM or all of it and its warps
+// meet at every exchange; 8 32 32 and 16 32 32 take two exchanges where 2 16 16 16
+// and 4 16 16 16 take three, for about as many instructions.  Measured per 2^26
+// points, radix 16 -> 32: 2^13 229 -> 202 us, 2^14 243 -> 212 (a copy takes
+// 158); range compression 355 -> 324 and 414 -> 373.  At 2^12 three radix-16
+// passes already take two exchanges (170 us).
 constexpr int row_lgm(int lg) { return lg >= 13 ? 5 : 4; }
 
 // Persistent TMA-staged variant of MAP_JJ (tile_fft_tma.cuh), one per length;
