@@ -12,13 +12,18 @@
 //     X[k] = E + W_N^k O,  E = (Z[k] + conj Z[M-k]) / 2,  O = (Z[k] - conj Z[M-k]) / (2i),
 // and M - k = (N1 - k1) + N1 (N2 - 1 - k2) lies in row N1 - k1 (row 0 and row
 // N1/2 are their own mirrors).  A tile of this kernel therefore takes H
-// mirror pairs of rows (8 for rows of up to 2^10 points, 4 for 2^11, 2 for
-// 2^12) -- rows u, u+1, ... and N1 - u, N1 - u - 1, ..., with rows 0 and N1/2
+// mirror pairs of rows (8 for rows of up to 2^9 points, 4 for 2^10 and 2^11, 2
+// for 2^12) -- rows u, u+1, ... and N1 - u, N1 - u - 1, ..., with rows 0 and N1/2
 // as the pair of u = 0 -- runs their 2H row FFTs with the same Stockham
 // passes as the row pass (tile_fft.cuh, last pass left in shared memory,
-// transposed so that a warp reads 2H rows at one k2 without bank conflicts),
-// and computes every X[k] of those rows from shared memory, stored as runs of
-// H consecutive k1 (8 bytes each).  X[M] comes from Z[0].
+// transposed), and one thread forms both X[k] and X[M - k] of a pair: one read
+// of each Z, one factor and one E and O for two outputs, stored as runs of H
+// consecutive k1 (8 bytes each).  X[M] comes from Z[0].  The kernel is bound
+// inside the SM; a thread that formed one output read two Z and a factor for
+// each.  Measured per 2^26 reals on GB300, both passes, one -> two outputs a
+// thread (a copy twice takes 158 us): 2^16 199 -> 185, 2^18 253 -> 239 (4 pairs
+// of rows a tile instead of 8, three tiles an SM instead of one: 229), 2^20
+// 278 -> 250, 2^22 321 -> 280.
 #include <cuda_runtime.h>
 
 #include "gbfft_internal.h"
@@ -27,9 +32,9 @@
 
 namespace gbfft {
 
-// Mirror pairs of rows per tile: 8 for rows of 2^6..2^10 points, fewer for
-// longer rows so that the tile fits shared memory (rows of 2^11: 4, 2^12: 2).
-constexpr int fold_pairs(int lg2) { return lg2 <= 10 ? 8 : (lg2 == 11 ? 4 : 2); }
+// Mirror pairs of rows per tile: 8 for rows of 2^6..2^9 points, fewer for longer
+// rows so that three tiles of 2^10-point rows, or one of 2^12, fit an SM.
+constexpr int fold_pairs(int lg2) { return lg2 <= 9 ? 8 : (lg2 <= 11 ? 4 : 2); }
 
 struct RFoldArgs {
   long long M;             // complex length (N / 2)
@@ -74,32 +79,48 @@ __global__ void __launch_bounds__(FoldCfg<LG2>::T) r2c_fold_kernel(const TileArg
   float2 v[Cfg::Tile::P];
   tile_stage<LG2, C, false, false, 0, true, 0, 6>(v, smem, a, ta.in + b * ta.in_bstride, nullptr, 0, b, nullptr);
 
-  // every Z of the C rows is in shared memory, Z_c[k2] at k2 * (C + 1) + c
+  // Every Z of the C rows is in shared memory, Z_c[k2] at k2 * (C + 1) + c.  One
+  // thread takes a mirror pair: Z[k] of row c < H and Z[M - k] of row c + H give
+  // X[k] and X[M - k] = conj(E - W O).  H lanes are a run of H k1; the 16 / H runs
+  // of a half warp are H elements k2 apart, which puts them on different banks.
   float2* xr = ta.out + b * (f.M + 1);
   const unsigned lo_mask = (1u << f.r_s) - 1u;
-  for (int idx = threadIdx.x; idx < C * N2; idx += T) {
-    const int c = idx & (C - 1), k2 = idx / C;
-    const int k1 = s_k1[c];
-    const bool self = (g == 0 && (c & (H - 1)) == 0);   // rows 0 and N1/2 mirror themselves
-    const int pc = self ? c : (c ^ H);
-    const int pk2 = (k1 == 0) ? ((N2 - k2) & (N2 - 1)) : (N2 - 1 - k2);
-    const float2 zk = smem[k2 * (C + 1) + c];
-    const float2 zm = smem[pk2 * (C + 1) + pc];
-    const unsigned k = (unsigned)k1 + (unsigned)f.N1 * (unsigned)k2;
+  const float s_int = f.scale ? f.s_int : 1.f;
+  const int c = threadIdx.x & (H - 1), k1 = s_k1[c];
+  const bool self = g == 0 && c == 0;   // rows 0 and N1/2 mirror themselves
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < H * N2; idx += T) {
+    const int i16 = idx >> 4, k2 = (idx & 15 & ~(H - 1)) + i16 % H + (i16 / H << 4);
+    int ck = c, row = k1, m2 = k2, p2 = N2 - 1 - k2;
+    int cm = c + H;
+    if (self) {
+      // elements 1..N2/2 are the pairs (k2, N2 - k2) of row 0, the others the
+      // pairs (k2, N2 - 1 - k2) of row N1/2
+      if (k2 >= 1 && k2 <= N2 / 2) {
+        cm = 0;
+        p2 = N2 - k2;
+      } else {
+        ck = H;
+        row = f.N1 / 2;
+        m2 = k2 == 0 ? 0 : k2 - N2 / 2;
+        p2 = N2 - 1 - m2;
+      }
+      if (k2 == 0) {   // X[0] and X[M] from Z[0]
+        const float2 z = smem[0];
+        const float s_end = f.scale ? f.s_end : 1.f;
+        __stcs(xr, make_float2((z.x + z.y) * s_end, 0.f));
+        __stcs(xr + f.M, make_float2((z.x - z.y) * s_end, 0.f));
+      }
+    }
+    const float2 zk = smem[m2 * (C + 1) + ck];
+    const float2 zm = smem[p2 * (C + 1) + cm];
+    const unsigned k = (unsigned)row + (unsigned)f.N1 * (unsigned)m2;
     const float2 w = cmul(__ldg(f.r_lo + (k & lo_mask)), __ldg(f.r_hi + (k >> f.r_s)));
     const float2 e = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
     const float2 o = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-    float2 x = cadd(e, cmul(w, o));
-    if (f.scale) {
-      const float sc = k == 0 ? f.s_end : f.s_int;
-      x = make_float2(x.x * sc, x.y * sc);
-    }
-    __stcs(xr + k, x);
-    if (k == 0) {
-      // X[M] = E[0] - O[0] (W_N^M = -1), real
-      const float xm = zk.x - zk.y;
-      __stcs(xr + f.M, make_float2(f.scale ? xm * f.s_end : xm, 0.f));
-    }
+    const float2 wo = cmul(w, o);
+    __stcs(xr + k, make_float2((e.x + wo.x) * s_int, (e.y + wo.y) * s_int));
+    __stcs(xr + (f.M - k), make_float2((e.x - wo.x) * s_int, (wo.y - e.y) * s_int));
   }
 }
 

@@ -91,8 +91,8 @@ const TileKernelInfo* tile_kernel_jc_b(int lg, int C);
 // (two passes, one exchange, where radix 16 takes three and two).  Measured per
 // 2^26 points: 1024 x 1024 images 384 -> 350 us, 2^26 582 -> 561; 2^20's row
 // pass at a copy's rate.  (Fewer columns leave too few threads a CTA; the real
-// rows folded into a 2^10-point row pass, one CTA of 16 rows per SM, measured
-// slower: rfft of 2^18 259 -> 267.)
+// rows folded into a 2^10-point row pass measure the same with either radix:
+// rfft of 2^18 229 and 230 us.)
 #define GBFFT_TK32(LG, C, ICF, OCF, MAP)                                                               \
   {(const void*)&tile_fft_kernel<LG, C, ICF, OCF, 5>, TileCfg<LG, C, ICF, OCF, 0, 5>::T,                \
    TileCfg<LG, C, ICF, OCF, 0, 5>::SMEM_BYTES, LG, C, MAP, 5}
