@@ -13,11 +13,12 @@ namespace gbfft {
 
 using namespace mixr;
 
-// contiguous transforms (0_) or strided columns (1_), any pad (_0) or evenly spaced (_1)
-const void* fx_fn_0_0();
-const void* fx_fn_0_1();
-const void* fx_fn_1_0();
-const void* fx_fn_1_1();
+// contiguous transforms (0_) or strided columns (1_), any pad (_0) or evenly spaced (_1);
+// only: N is a single radix
+const void* fx_fn_0_0(bool only);
+const void* fx_fn_0_1(bool only);
+const void* fx_fn_1_0(bool only);
+const void* fx_fn_1_1(bool only);
 
 static unsigned recip(unsigned d) { return d == 1 ? 0u : (unsigned)((0x100000000ULL + d - 1) / d); }
 
@@ -99,7 +100,8 @@ int fx_init(FxLaunch& L, long long N, long long ncols, long long batches, const 
     a.st_st[s] = (n1 + (pad ? n1 >> 4 : 0)) * unit;
   }
   L.threads = best.T;
-  L.fn = lay ? (lin ? fx_fn_1_1() : fx_fn_1_0()) : (lin ? fx_fn_0_1() : fx_fn_0_0());
+  const bool only = a.nrad == 1;
+  L.fn = lay ? (lin ? fx_fn_1_1(only) : fx_fn_1_0(only)) : (lin ? fx_fn_0_1(only) : fx_fn_0_0(only));
   if (L.smem > 48 * 1024 &&
       cudaFuncSetAttribute(L.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess)
     return FFT_ERR_CUDA;

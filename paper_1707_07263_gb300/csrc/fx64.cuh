@@ -589,41 +589,43 @@ __device__ __noinline__ void fx_special_tile(const FxTile<STR, LIN>& T) {
     default: CALL(16); break;    \
   }
 
-// 128 registers: one CTA of 512 threads per SM, two of 256, four of 128.
 template <bool STR, bool LIN>
-__global__ void __launch_bounds__(512, 1) fx_kernel(const FxArgs a) {
-  extern __shared__ __align__(16) unsigned char fx_smem[];
+__device__ __forceinline__ FxTile<STR, LIN> fx_tile(const FxArgs& a, unsigned char* smem) {
   const long long t = a.tile0 + blockIdx.x;
-  const double2* gin;
-  double2* gout;
-  unsigned col0 = 0;
-  int valid;
   if constexpr (STR) {
     const long long bt = t / a.tiles_per_batch;
     const long long c0 = (t - bt * a.tiles_per_batch) << a.csh;
-    col0 = (unsigned)c0;
-    valid = (int)(a.ncols - c0 < a.C ? a.ncols - c0 : a.C);
-    gin = a.in + bt * a.in_bs + c0 * a.in_cs;
-    gout = a.out + bt * a.out_bs + c0 * a.out_cs;
+    const int valid = (int)(a.ncols - c0 < a.C ? a.ncols - c0 : a.C);
+    return FxTile<STR, LIN>{a, (Fx*)smem, (int*)(smem + a.slot_off), a.in + bt * a.in_bs + c0 * a.in_cs,
+                            a.out + bt * a.out_bs + c0 * a.out_cs, (unsigned)c0, valid};
   } else {
     const long long c0 = t * a.C;
-    valid = (int)(a.ncols - c0 < a.C ? a.ncols - c0 : a.C);
-    gin = a.in + c0 * a.N;
-    gout = a.out + c0 * a.N;
+    const int valid = (int)(a.ncols - c0 < a.C ? a.ncols - c0 : a.C);
+    return FxTile<STR, LIN>{a, (Fx*)smem, (int*)(smem + a.slot_off), a.in + c0 * a.N, a.out + c0 * a.N, 0u, valid};
   }
-  int* slot = (int*)(fx_smem + a.slot_off);
-  const FxTile<STR, LIN> T{a, (Fx*)fx_smem, slot, gin, gout, col0, valid};
+}
+
+// N is a single radix (at most 7).  A kernel of its own: inside fx_kernel these
+// branches cost every length 2,268 bytes of spills (4096 points: @@).
+template <bool STR, bool LIN>
+__global__ void __launch_bounds__(256) fx_only_kernel(const __grid_constant__ FxArgs a) {
+  const FxTile<STR, LIN> T = fx_tile<STR, LIN>(a, nullptr);
+  switch (a.rad[0]) {
+    case 2: T.template only<2>(); break;
+    case 3: T.template only<3>(); break;
+    case 4: T.template only<4>(); break;
+    case 5: T.template only<5>(); break;
+    default: T.template only<7>(); break;
+  }
+}
+
+// 128 registers: one CTA of 512 threads per SM, two of 256, four of 128.
+template <bool STR, bool LIN>
+__global__ void __launch_bounds__(512, 1) fx_kernel(const __grid_constant__ FxArgs a) {
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  const FxTile<STR, LIN> T = fx_tile<STR, LIN>(a, fx_smem);
+  int* const slot = T.slot;
   const int last = a.nrad - 1;
-  if (last == 0) {
-    switch (a.rad[0]) {
-      case 2: T.template only<2>(); break;
-      case 3: T.template only<3>(); break;
-      case 4: T.template only<4>(); break;
-      case 5: T.template only<5>(); break;
-      default: T.template only<7>(); break;
-    }
-    return;
-  }
   for (int i = threadIdx.x; i < a.nrad * a.C; i += blockDim.x) slot[i] = 0;
   __syncthreads();
   bool special = false;

@@ -2,5 +2,7 @@
 #include "fx64.cuh"
 
 namespace gbfft {
-const void* fx_fn_0_0() { return (const void*)fx_kernel<false, false>; }
+const void* fx_fn_0_0(bool only) {
+  return only ? (const void*)fx_only_kernel<false, false> : (const void*)fx_kernel<false, false>;
+}
 }  // namespace gbfft

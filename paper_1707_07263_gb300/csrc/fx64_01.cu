@@ -2,5 +2,7 @@
 #include "fx64.cuh"
 
 namespace gbfft {
-const void* fx_fn_0_1() { return (const void*)fx_kernel<false, true>; }
+const void* fx_fn_0_1(bool only) {
+  return only ? (const void*)fx_only_kernel<false, true> : (const void*)fx_kernel<false, true>;
+}
 }  // namespace gbfft

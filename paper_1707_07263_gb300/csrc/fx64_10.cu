@@ -2,5 +2,7 @@
 #include "fx64.cuh"
 
 namespace gbfft {
-const void* fx_fn_1_0() { return (const void*)fx_kernel<true, false>; }
+const void* fx_fn_1_0(bool only) {
+  return only ? (const void*)fx_only_kernel<true, false> : (const void*)fx_kernel<true, false>;
+}
 }  // namespace gbfft

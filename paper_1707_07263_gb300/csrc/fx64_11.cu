@@ -2,5 +2,7 @@
 #include "fx64.cuh"
 
 namespace gbfft {
-const void* fx_fn_1_1() { return (const void*)fx_kernel<true, true>; }
+const void* fx_fn_1_1(bool only) {
+  return only ? (const void*)fx_only_kernel<true, true> : (const void*)fx_kernel<true, true>;
+}
 }  // namespace gbfft
