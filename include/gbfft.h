@@ -92,9 +92,9 @@ enum {
  * or (FP32 and FP64) a product n = 2^a 3^b 5^c 7^d (mixed radix: Eq. 1 holds
  * for any n and the Cooley-Tukey split of Sec. 2.1 for any factorisation;
  * a config must be NULL).  Mixed-radix lengths up to 14336 run as one on-chip
- * pass of radix-16/8/4/2/3/5/7 stages; longer ones, up to 14336^2, as the
- * four-step split n = N1 N2 (N1 the largest divisor of n at most sqrt(n)
- * whose cofactor N2 is at most 14336): a strided column pass with the twiddle
+ * pass of stages of 2 to 25 points; longer ones, up to 14336^2, as the
+ * four-step split n = N1 N2 (both at most 14336; the split whose two passes
+ * the plan's cost model prefers): a strided column pass with the twiddle
  * W_n^{n2 k1}, then a row pass, through a workspace (fft_plan_kind 6).  A
  * 7-smooth n with no such split, or beyond 14336^2, gives FFT_ERR_UNSUPPORTED.
  * FP64 plans take the same routes with 7168 in place of 14336, for powers of
@@ -142,10 +142,10 @@ GBFFT_API fft_plan* fft_plan_create_2d(int64_t ny, int64_t nx, int64_t batch, in
  * The row of n reals is read as n/2 complex values x[2m] + i x[2m+1] (Sec. 2.1
  * splits a sequence into even and odd samples the same way); one complex
  * transform of length n/2 and one split step give the result.  n <= 2^15: one
- * fused kernel, one read and one write of every value.  2^16 <= n <= 2^22,
+ * fused kernel, one read and one write of every value.  2^16 <= n <= 2^23,
  * real to complex: the complex plan's column pass, then its row pass with the
  * split folded in (rows k1 and n/2/N1 - k1 in one tile), two passes.
- * 2^16 <= n <= 2^21, complex to real: the split folded into the complex
+ * The same lengths, complex to real: the split folded into the complex
  * plan's column pass (X[m] and X[n/2 - m] read from the same row), then its
  * row pass, two passes.  Other longer n and directions: the complex plan plus
  * one split kernel.  Multi-pass lengths need a workspace

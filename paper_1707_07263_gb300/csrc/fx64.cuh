@@ -18,20 +18,21 @@
 //   * the last pass turns integers back into FP64, rounded to nearest.
 // The largest value of a transform holds 57 to 62 bits at all times, against
 // 53 in FP64, and factors are right to 2^-62.  Measured error (relative L2
-// against 113-bit arithmetic, 13 lengths from 6 to 32768; Gaussian, uniform,
+// against 113-bit arithmetic, 16 lengths from 6 to 2^20; Gaussian, uniform,
 // impulses, sparse, 26 decades of dynamic range, tones, smooth and whole-number
-// rows): 0.17 to 1.0 of the FP64 kernel's that this replaced (4096 points,
+// rows): 0.13 to 1.0 of the FP64 kernel's that this replaced (4096 points,
 // Gaussian: 5.9e-17 against 2.3e-16).
 // Every transform has its own exponent.  One that holds an infinity or a NaN
 // takes its tile through plain FP64 sums (fx_special_tile); results outside
 // FP64's normal range take scalbn's rounding to subnormal numbers, zero or
 // infinity.
-// Radix 16 with 16 points a thread (128 registers, 16 warps an SM) issues about
-// 40 % of the time at 4096 points, held by latency and instruction fetch; radix
-// 8 with 64 registers takes one pass more and measured 407 us against 305.
-// Measured per 2^24 points on GB300, against the FP64 kernel: 64 641 -> 203 us,
-// 1000 1463 -> 387, 4096 1348 -> 294, 7000 1880 -> 667; two passes: 65536
-// 1961 -> 483, 2^20 2485 -> 719.
+// Radix 16 with 16 points a thread (128 registers): 16 warps an SM, held by
+// latency and instruction fetch; radix 8 at the same 16 points and warps takes
+// one pass more (290 against 254 us per 2^24 points at 4096), with 64 registers
+// and 32 warps it spills as well (407 against 305, an earlier form).
+// Measured per 2^24 points on GB300, against the FP64 kernel: 64 641 -> 146 us,
+// 1000 1463 -> 317, 4096 1348 -> 230, 7000 1880 -> 541; two passes: 65536
+// 1961 -> 366, 2^20 2485 -> 545.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -606,7 +607,8 @@ __device__ __forceinline__ FxTile<STR, LIN> fx_tile(const FxArgs& a, unsigned ch
 }
 
 // N is a single radix (at most 7).  A kernel of its own: inside fx_kernel these
-// branches cost every length 2,268 bytes of spills (4096 points: @@).
+// branches cost the others 2,268 bytes of spills, 81 local stores and 91 loads a
+// thread at 4096 points (294 us per 2^24 points against 230).
 template <bool STR, bool LIN>
 __global__ void __launch_bounds__(256) fx_only_kernel(const __grid_constant__ FxArgs a) {
   const FxTile<STR, LIN> T = fx_tile<STR, LIN>(a, nullptr);

@@ -77,8 +77,8 @@ inline float pass_cost_f32(int r, bool first, bool last, bool pad) {
   return per;
 }
 // The same for the 64-bit fixed-point passes: a fit to 6,700 measured
-// (schedule, columns, threads) of 29 lengths from 60 to 7168 (pick 1.9 % slower
-// than the fastest measured on average, at most 12 %).
+// (schedule, columns, threads) of 29 lengths from 60 to 7168 (the pick is 2 %
+// slower than the fastest measured on average, at most 7 %).
 inline float pass_cost_fx(int r, bool first, bool last, bool) {
   const float dft = r == 2 ? 3.5f : r == 3 ? 8.f : r == 4 ? 15.5f : r == 5 ? 27.2f : r == 7 ? 37.5f
                     : r == 8 ? 25.4f : r == 9 ? 36.3f : r == 10 ? 55.8f : r == 12 ? 33.f : r == 14 ? 56.9f

@@ -1,5 +1,5 @@
 // real_fold.cu -- real-data transforms of N = 2M reals with M = N1 * N2 a
-// two-pass four-step length (2^15..2^21): the even/odd split folded into the
+// two-pass four-step length (2^15..2^22): the even/odd split folded into the
 // row pass of the complex transform (real to complex) or into its column pass
 // (complex to real), so that the transform takes two passes over memory
 // instead of three.
