@@ -62,9 +62,14 @@ enum {
   FFT_PREC_TC_FP16 = 2,
   FFT_PREC_TC_BF16_SPLIT = 3,
   FFT_PREC_TC_FP16_SPLIT = 4,
-  /* complex128 data; arithmetic in 64-bit integers with one exponent per
-   * sub-transform (its largest value holds 57 to 62 bits), more exact than FP64
-   * sums over a transform, infinities and NaN in FP64; 1-D plans of 7-smooth length
+  /* complex128 data.  A transform whose inputs are of one scale runs in 64-bit
+   * integers with one exponent (its largest value holds 57 to 62 bits): the error
+   * against the norm of its row is below that of FP64 sums, but an input below
+   * about 2^-57 of the row's largest counts only as far as it carries into that
+   * unit, which shows where larger inputs cancel exactly.  Transforms whose real
+   * or imaginary parts, or some of whose first sums, lie at another scale, and
+   * those with infinities or NaN, run in FP64 arithmetic, at about a fifth of the
+   * speed; one transform's choice does not touch another's.  1-D plans of 7-smooth length
    * n = 2^a 3^b 5^c 7^d (powers of two included): one on-chip pass for
    * 2 <= n <= 7168, two strided passes (four-step, workspace) for
    * 7168 < n <= 7168^2 when n = N1 N2 with N1, N2 <= 7168 (powers of two up

@@ -23,7 +23,7 @@ const void* fx_fn_1_1(bool only);
 static unsigned recip(unsigned d) { return d == 1 ? 0u : (unsigned)((0x100000000ULL + d - 1) / d); }
 
 // Entries of the plan's tables: the twiddles of every pass after the first,
-// then W_N^m for the FP64 fallback.
+// then W_N^m for FP64 arithmetic.
 size_t fx_table_entries(const FxArgs& a) {
   size_t n = (size_t)a.N;
   for (int s = 1; s < a.nrad; ++s) n += (size_t)(a.rad[s] - 1) * a.ns[s];
@@ -35,9 +35,8 @@ int fx_fill_tables(FxLaunch& L, int4* tab, cudaStream_t s) {
   a.tw = tab;
   for (int i = 1; i < a.nrad; ++i)
     if (launch_gen_fx_twiddles(tab + a.tw_off[i], a.rad[i], (int)a.ns[i], s) != cudaSuccess) return FFT_ERR_CUDA;
-  int4* wn = tab + fx_table_entries(a) - a.N;
-  a.wn = wn;
-  return launch_gen_fx_power(wn, a.N, a.N, 1, s) == cudaSuccess ? FFT_OK : FFT_ERR_CUDA;
+  a.wn = (const double2*)(tab + fx_table_entries(a) - a.N);
+  return launch_gen_twiddles_step((void*)a.wn, true, a.N, a.N, 1, s) == cudaSuccess ? FFT_OK : FFT_ERR_CUDA;
 }
 
 // Fills L for `batches` batches of ncols sub-transforms of length N

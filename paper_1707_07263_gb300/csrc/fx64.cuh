@@ -17,30 +17,36 @@
 //     is the headroom the next additions need anyway;
 //   * the last pass turns integers back into FP64, rounded to nearest.
 // The largest value of a transform holds 57 to 62 bits at all times, against
-// 53 in FP64, and factors are right to 2^-62.  Measured error (relative L2
-// against 113-bit arithmetic, 16 lengths from 6 to 2^20; Gaussian, uniform,
-// impulses, sparse, 26 decades of dynamic range, tones, smooth and whole-number
-// rows): 0.13 to 1.0 of the FP64 kernel's that this replaced (4096 points,
-// Gaussian: 5.9e-17 against 2.3e-16).
-// Every transform has its own exponent.  One that holds an infinity or a NaN
-// takes its tile through plain FP64 sums (fx_special_tile); results outside
-// FP64's normal range take scalbn's rounding to subnormal numbers, zero or
-// infinity.
+// 53 in FP64, and factors are right to 2^-62, so the error against the norm of a
+// row is below that of FP64 sums (4096 points, Gaussian: 5.9e-17 against 2.3e-16).
+// Values far below a row's largest have fewer bits, though, where FP64 has 53 at
+// any size.  Each transform is therefore looked at as it is read
+// (FxTile::wide, fx_plane_bits): those whose inputs are not of one scale, those
+// that hold an infinity or a NaN, and those between normal and subnormal numbers
+// run in FP64 arithmetic instead, after the tile's other columns
+// (fx_mixed_tile; a tile of such transforms alone 1546 us at 4096 points, 2500 at
+// 7000).  The choice is a transform's own:
+// its neighbours in the tile do not change it.  Results outside FP64's normal
+// range take scalbn's rounding to subnormal numbers, zero or infinity.
 // Radix 16 with 16 points a thread (128 registers): 16 warps an SM, held by
 // latency and instruction fetch; radix 8 at the same 16 points and warps takes
 // one pass more (290 against 254 us per 2^24 points at 4096), with 64 registers
 // and 32 warps it spills as well (407 against 305, an earlier form).
-// Measured per 2^24 points on GB300, against the FP64 kernel: 64 641 -> 146 us,
-// 1000 1463 -> 317, 4096 1348 -> 230, 7000 1880 -> 541; two passes: 65536
+// Measured per 2^24 points on GB300, against the FP64 kernel: 64 641 -> 151 us,
+// 1000 1463 -> 321, 4096 1348 -> 234, 7000 1880 -> 545; two passes: 65536
 // 1961 -> 366, 2^20 2485 -> 545.
 #pragma once
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "fx64_math.h"
 #include "gbfft_internal.h"
 #include "mixed_common.cuh"
 
 namespace gbfft {
+
+constexpr double k2m62 = 2.168404344971008868e-19;   // 2^-62
 
 // ---- DFTs ------------------------------------------------------------------------
 __device__ __forceinline__ long long fx_shl(long long x, int s) { return (long long)((unsigned long long)x << s); }
@@ -91,21 +97,50 @@ __device__ __forceinline__ Fx fx_mulw(Fx a) {
   }
 }
 
-__device__ __forceinline__ void fx_dft2(Fx& a, Fx& b) {
-  const Fx t = a;
+// The same in FP64, for the transforms that fixed point would shorten.
+__device__ __forceinline__ double2 fx_add(double2 a, double2 b) { return gadd(a, b); }
+__device__ __forceinline__ double2 fx_sub(double2 a, double2 b) { return gsub(a, b); }
+template <int R, int M>
+__device__ __forceinline__ double2 fx_mulw(double2 a) {
+  constexpr int m = M % R;
+  if constexpr (m == 0) {
+    return a;
+  } else if constexpr ((4 * m) % R == 0) {
+    constexpr int qt = 4 * m / R;
+    if constexpr (qt == 1) return make_double2(a.y, -a.x);
+    else if constexpr (qt == 2) return make_double2(-a.x, -a.y);
+    else return make_double2(-a.y, a.x);
+  } else if constexpr ((8 * m) % R == 0) {
+    constexpr int et = 8 * m / R;
+    constexpr double r2 = (double)fx_cossin(1, 8).c * k2m62;
+    const double p = r2 * (a.x + a.y), d = r2 * (a.y - a.x);
+    if constexpr (et == 1) return make_double2(p, d);
+    else if constexpr (et == 3) return make_double2(d, -p);
+    else if constexpr (et == 5) return make_double2(-p, -d);
+    else return make_double2(-d, p);
+  } else {
+    constexpr double c = (double)fx_cossin(m, R).c * k2m62, s = (double)fx_cossin(m, R).s * k2m62;
+    return gmul(a, make_double2(c, -s));
+  }
+}
+
+template <typename V>
+__device__ __forceinline__ void fx_dft2(V& a, V& b) {
+  const V t = a;
   a = fx_add(t, b);
   b = fx_sub(t, b);
 }
-__device__ __forceinline__ void fx_dft4(Fx& x0, Fx& x1, Fx& x2, Fx& x3) {
-  const Fx t0 = fx_add(x0, x2), t1 = fx_sub(x0, x2), t2 = fx_add(x1, x3), d = fx_sub(x1, x3);
+template <typename V>
+__device__ __forceinline__ void fx_dft4(V& x0, V& x1, V& x2, V& x3) {
+  const V t0 = fx_add(x0, x2), t1 = fx_sub(x0, x2), t2 = fx_add(x1, x3), d = fx_sub(x1, x3);
   x0 = fx_add(t0, t2);
   x2 = fx_sub(t0, t2);
-  x1 = Fx{t1.x + d.y, t1.y - d.x};
-  x3 = Fx{t1.x - d.y, t1.y + d.x};
+  x1 = V{t1.x + d.y, t1.y - d.x};
+  x3 = V{t1.x - d.y, t1.y + d.x};
 }
 
-template <int R>
-__device__ __forceinline__ void fx_dft(Fx* v);
+template <int R, typename V>
+__device__ __forceinline__ void fx_dft(V* v);
 
 // odd primes, as dft_odd of mixed_common.cuh
 template <int R, int k, int m>
@@ -148,8 +183,8 @@ __device__ __forceinline__ void fx_dft_odd(Fx* v) {
   for (int q = 0; q < R; ++q) v[q] = out[q];
 }
 
-template <int R, int B, int n2, int k1, int A>
-__device__ __forceinline__ void fx_inner(Fx (&x)[B][A]) {
+template <int R, int B, int n2, int k1, int A, typename V>
+__device__ __forceinline__ void fx_inner(V (&x)[B][A]) {
   if constexpr (n2 < B) {
     if constexpr (k1 < A) {
       x[n2][k1] = fx_mulw<R, n2 * k1>(x[n2][k1]);
@@ -160,10 +195,10 @@ __device__ __forceinline__ void fx_inner(Fx (&x)[B][A]) {
   }
 }
 // R = A B, as ct_dft_split of mixed_ct.cuh
-template <int A, int B>
-__device__ __forceinline__ void fx_dft_split(Fx* v) {
+template <int A, int B, typename V>
+__device__ __forceinline__ void fx_dft_split(V* v) {
   constexpr int R = A * B;
-  Fx x[B][A];
+  V x[B][A];
 #pragma unroll
   for (int n2 = 0; n2 < B; ++n2)
 #pragma unroll
@@ -171,7 +206,7 @@ __device__ __forceinline__ void fx_dft_split(Fx* v) {
 #pragma unroll
   for (int n2 = 0; n2 < B; ++n2) fx_dft<A>(x[n2]);
   fx_inner<R, B, 1, 1, A>(x);
-  Fx y[A][B];
+  V y[A][B];
 #pragma unroll
   for (int k1 = 0; k1 < A; ++k1)
 #pragma unroll
@@ -184,10 +219,11 @@ __device__ __forceinline__ void fx_dft_split(Fx* v) {
     for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = y[k1][k2];
 }
 
-template <int R>
-__device__ __forceinline__ void fx_dft(Fx* v) {
+template <int R, typename V>
+__device__ __forceinline__ void fx_dft(V* v) {
   if constexpr (R == 2) fx_dft2(v[0], v[1]);
   else if constexpr (R == 4) fx_dft4(v[0], v[1], v[2], v[3]);
+  else if constexpr ((R == 3 || R == 5 || R == 7) && std::is_same_v<V, double2>) dft_odd<R>(v);
   else if constexpr (R == 3 || R == 5 || R == 7) fx_dft_odd<R>(v);
   else if constexpr (R == 8) fx_dft_split<4, 2>(v);
   else if constexpr (R == 9) fx_dft_split<3, 3>(v);
@@ -223,9 +259,8 @@ static __device__ __noinline__ double fx_out_any(long long q, int ex) { return s
 // a Q62 table factor in FP64
 __device__ __forceinline__ double2 fx_factor(const int4* p) {
   const Cq62 w = fx_ldw(p);
-  const double s = 2.168404344971008868e-19;   // 2^-62
-  return make_double2(((double)w.r.h * 4294967296.0 + (double)w.r.l) * s,
-                      ((double)w.i.h * 4294967296.0 + (double)w.i.l) * s);
+  return make_double2(((double)w.r.h * 4294967296.0 + (double)w.r.l) * k2m62,
+                      ((double)w.i.h * 4294967296.0 + (double)w.i.l) * k2m62);
 }
 
 // points a thread holds in the first and the middle passes: with 20, two
@@ -303,19 +338,22 @@ struct FxTile {
     return e;
   }
 
+  // with the largest high words of the real and the imaginary parts
   template <int R>
-  __device__ __forceinline__ void load_bits(double2* v, int c, int j, int NB, int& top) const {
+  __device__ __forceinline__ void load_bits(double2* v, int c, int j, int NB, int& tx, int& ty) const {
     const bool ok = c < valid;
+    tx = ty = 0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       v[r] = ok ? __ldcs(in_at(c, j + r * NB)) : make_double2(0, 0);
-      top = max(top, max(__double2hiint(v[r].x) & 0x7fffffff, __double2hiint(v[r].y) & 0x7fffffff));
+      tx = max(tx, __double2hiint(v[r].x) & 0x7fffffff);
+      ty = max(ty, __double2hiint(v[r].y) & 0x7fffffff);
     }
   }
   template <int R>
   __device__ __forceinline__ void to_fixed(Fx* f, const double2* v, int E) const {
     constexpr int F = 62 - fx_headroom(R);
-    if (E > 64) {
+    if (E > kFxSubnormal) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         f[r].x = fx_from_bits<false>(__double_as_longlong(v[r].x), E, F);
@@ -404,38 +442,64 @@ struct FxTile {
     }
   }
 
-  // True (for the whole CTA) when the tile holds an infinity or a NaN: then
-  // nothing was done.
+  // Whether fixed point would shorten a butterfly's inputs beside the row's
+  // largest high word top (fx_plane_bits); tx and ty as load_bits gives them.
+  template <int R>
+  __device__ __forceinline__ bool wide(const double2* v, int tx, int ty, int top) const {
+    const int E = fx_row_exponent(top);
+    if (E <= 64) return E > kFxSubnormal;
+    const int least = top - (fx_plane_bits(R) << 20);
+    if (min(tx, ty) >= least) return false;
+    if ((tx > 0 && tx < least) || (ty > 0 && ty < least)) return true;
+    int low = 0;   // zeros lose nothing, but numbers whose high word is zero would
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      low |= __double2hiint(v[r].x) & 0x7fffffff ? 0 : __double2loint(v[r].x);
+      low |= __double2hiint(v[r].y) & 0x7fffffff ? 0 : __double2loint(v[r].y);
+    }
+    return low != 0;
+  }
+  // The transform of column c is left to FP64 arithmetic.
+  __device__ __forceinline__ bool in_fp64(int c) const { return slot[c] >= 0x7ff00000; }
+
+  // True in a thread that met a column for FP64 arithmetic.
   template <int R, int K>
   __device__ __forceinline__ bool first() const {
     const int NB = (int)a.nb[0], total = a.C * NB;
     double2 v[K][R];
-    int special = 0;
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-      const int b = threadIdx.x + i * blockDim.x;
-      if (b < total) {
-        int c, j, top = 0;
-        split(b, 0, c, j);
-        load_bits<R>(v[i], c, j, NB, top);
-        special |= top >= 0x7ff00000;
-        atomicMax(slot + c, top);
-      }
-    }
-    if (__syncthreads_or(special)) return true;
+    int tx[K], ty[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
       const int b = threadIdx.x + i * blockDim.x;
       if (b < total) {
         int c, j;
         split(b, 0, c, j);
+        load_bits<R>(v[i], c, j, NB, tx[i], ty[i]);
+        atomicMax(slot + c, max(tx[i], ty[i]));
+      }
+    }
+    __syncthreads();
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const int b = threadIdx.x + i * blockDim.x;
+      if (b < total) {
+        int c, j;
+        split(b, 0, c, j);
+        const int top = slot[c];
+        if (top >= 0x7ff00000) {
+          any = true;
+        } else if (wide<R>(v[i], tx[i], ty[i], top)) {
+          atomicMax(slot + c, 0x7fffffff);
+          any = true;
+        }
         Fx f[R];
-        to_fixed<R>(f, v[i], fx_row_exponent(slot[c]));
+        to_fixed<R>(f, v[i], fx_row_exponent(top));
         fx_dft<R>(f);
         store_tile<R>(f, 0, c, j * R, 1);
       }
     }
-    return false;
+    return any;
   }
 
   template <int R, int K>
@@ -466,12 +530,14 @@ struct FxTile {
     }
   }
 
-  template <int R>
+  // SKIP: but the columns left to FP64 arithmetic
+  template <int R, bool SKIP>
   __device__ __forceinline__ void last(int s) const {
     const int NB = (int)a.nb[s], total = a.C * NB;   // Ns == NB
     for (int b = threadIdx.x; b < total; b += blockDim.x) {
       int c, j;
       split(b, s, c, j);
+      if (SKIP && in_fp64(c)) continue;
       Fx v[R];
       load_tile<R>(v, s, c, j, NB);
       rotate<R>(v, s, c, NB, j);
@@ -480,27 +546,45 @@ struct FxTile {
     }
   }
 
-  // N is a single radix (at most 7): one butterfly a transform, in registers
+  // N is a single radix (at most 7): one butterfly a transform, in registers.
+  // Radices 2 and 4 add in FP64, exact where the numbers are (180 and 242 us per
+  // 2^24 points; the integers take 127 and 124), but rows of subnormal numbers,
+  // which the integers hold exactly.
   template <int R>
   __device__ __forceinline__ void only() const {
     for (int c = threadIdx.x; c < a.C; c += blockDim.x) {
       double2 v[R];
-      int top = 0;
-      load_bits<R>(v, c, 0, 1, top);
-      if (top >= 0x7ff00000) {
-        special_butterfly<R>(v, c);
-        continue;
+      int tx, ty;
+      load_bits<R>(v, c, 0, 1, tx, ty);
+      const int top = max(tx, ty), E = fx_row_exponent(top);
+      bool fp64;
+      if constexpr (R == 2 || R == 4) {
+        int bits = top;
+#pragma unroll
+        for (int r = 0; r < R; ++r) bits |= __double2loint(v[r].x) | __double2loint(v[r].y);
+        fp64 = E > kFxSubnormal || bits == 0;
+      } else {
+        fp64 = top >= 0x7ff00000 || wide<R>(v, tx, ty, top);
       }
-      Fx f[R];
-      const int E = fx_row_exponent(top);
-      to_fixed<R>(f, v, E);
-      fx_dft<R>(f);
-      store_global<R>(f, c, 0, 1, E - 1022 - (62 - fx_headroom(R)));
+      if (fp64) {
+        if (a.conj_in) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[r].y = -v[r].y;
+        }
+        fx_dft<R>(v);
+#pragma unroll
+        for (int q = 0; q < R; ++q) store_double(v[q], c, q);
+      } else {
+        Fx f[R];
+        to_fixed<R>(f, v, E);
+        fx_dft<R>(f);
+        store_global<R>(f, c, 0, 1, E - 1022 - (62 - fx_headroom(R)));
+      }
     }
   }
 
   // output k of column c in FP64 arithmetic: four-step factor, conjugation, scale
-  __device__ __forceinline__ void store_special(double2 y, int c, int k) const {
+  __device__ __forceinline__ void store_double(double2 y, int c, int k) const {
     if (c >= valid) return;
     if (STR && a.ft) {
       y = gmul(y, fx_factor(a.ft + (size_t)(unsigned)k * a.ft_cols + (col0 + c)));
@@ -510,69 +594,61 @@ struct FxTile {
     }
     *out_at(c, k) = make_double2(y.x * a.scale, y.y * (a.conj_out ? -a.scale : a.scale));
   }
-  template <int R>
-  __device__ __noinline__ void special_butterfly(const double2* v, int c) const {
-    for (int q = 0; q < R; ++q) {
-      double2 sum = make_double2(0, 0);
-      for (int r = 0; r < R; ++r) {
-        const double2 x = make_double2(v[r].x, a.conj_in ? -v[r].y : v[r].y);
-        const int m = r * q % R;
-        sum = gadd(sum, m ? gmul(x, fx_factor(a.wn + m)) : x);
+
+  // Pass s of the columns left to FP64 arithmetic.
+  template <int R, int K>
+  __device__ __forceinline__ void double_pass(int s) const {
+    const int NB = (int)a.nb[s], Ns = (int)a.ns[s], total = a.C * NB;
+    const bool first = s == 0, last = s == a.nrad - 1;
+    const int step = NB / Ns;   // W_{Ns R} = W_N^{N / (Ns R)}
+    double2* const ds = (double2*)sm;
+    // (a middle pass has one round: its inputs are all held before any output is written)
+#pragma unroll 1
+    for (int base = threadIdx.x; base - (int)threadIdx.x < total; base += K * (int)blockDim.x) {
+      double2 v[K][R];
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        const int b = base + i * (int)blockDim.x;
+        int c = 0, j = 0;
+        if (b < total) split(b, s, c, j);
+        if (b < total && c < valid && in_fp64(c)) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            v[i][r] = first ? __ldcs(in_at(c, j + r * NB)) : ds[at(c, j + r * NB)];
+            if (first && a.conj_in) v[i][r].y = -v[i][r].y;
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[i][r] = make_double2(0, 0);
+        }
       }
-      store_special(sum, c, q);
+      if (!first && !last) __syncthreads();
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        const int b = base + i * (int)blockDim.x;
+        int c = 0, j = 0;
+        if (b < total) split(b, s, c, j);
+        if (b < total && c < valid && in_fp64(c)) {
+          const int jq = (int)fdiv((unsigned)j, a.ns_m[s]);
+          const int k = j - jq * Ns;
+          if (!first) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[i][r] = gmul(v[i][r], __ldg(a.wn + r * k * step));
+          }
+          fx_dft<R>(v[i]);
+          const int m0 = jq * Ns * R + k;
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            if (last)
+              store_double(v[i][q], c, m0 + q * Ns);
+            else
+              ds[at(c, m0 + q * Ns)] = v[i][q];
+          }
+        }
+      }
     }
   }
 };
-
-// The tile in FP64 arithmetic, for inputs that hold an infinity or a NaN: the
-// same passes, every butterfly as plain sums over its inputs (the factors
-// W_N^m from the table wn), outputs held by the threads until all inputs have
-// been read.
-template <bool STR, bool LIN>
-__device__ __noinline__ void fx_special_tile(const FxTile<STR, LIN>& T) {
-  const FxArgs& a = T.a;
-  double2* sm = (double2*)T.sm;
-  double2 out[kFxPoints];
-  for (int s = 0; s < a.nrad; ++s) {
-    const int R = a.rad[s], NB = (int)a.nb[s], Ns = (int)a.ns[s], total = a.C * NB;
-    const bool first = s == 0, last = s == a.nrad - 1;
-    const int step = a.N / (Ns * R);
-    __syncthreads();
-    int n = 0;
-    for (int b = threadIdx.x; b < total; b += blockDim.x) {
-      int c, j;
-      T.split(b, s, c, j);
-      const int jq = j / Ns, k = j - jq * Ns;
-      for (int q = 0; q < R; ++q) {
-        double2 sum = make_double2(0, 0);
-        for (int r = 0; r < R; ++r) {
-          double2 x = make_double2(0, 0);
-          if (!first) {
-            x = sm[T.at(c, j + r * NB)];
-          } else if (c < T.valid) {
-            x = *T.in_at(c, j + r * NB);
-            if (a.conj_in) x.y = -x.y;
-          }
-          const unsigned m = (unsigned)r * (unsigned)(k + q * Ns) % (unsigned)(Ns * R);
-          sum = gadd(sum, m ? gmul(x, fx_factor(a.wn + m * step)) : x);
-        }
-        if (last)
-          T.store_special(sum, c, k + q * Ns);
-        else
-          out[n++] = sum;
-      }
-    }
-    if (last) return;
-    __syncthreads();
-    n = 0;
-    for (int b = threadIdx.x; b < total; b += blockDim.x) {
-      int c, j;
-      T.split(b, s, c, j);
-      const int jq = j / Ns, k = j - jq * Ns;
-      for (int q = 0; q < R; ++q) sm[T.at(c, jq * Ns * R + k + q * Ns)] = out[n++];
-    }
-  }
-}
 
 #define GBFFT_FX_SWITCH(r, CALL) \
   switch (r) {                   \
@@ -621,33 +697,59 @@ __global__ void __launch_bounds__(256) fx_only_kernel(const __grid_constant__ Fx
   }
 }
 
+// The passes in fixed point after the first.
+template <bool SKIP, bool STR, bool LIN>
+__device__ __forceinline__ void fx_passes(const FxTile<STR, LIN>& T) {
+  const int last = T.a.nrad - 1;
+  for (int s = 1; s < last; ++s) {
+#define CALL(R) T.template middle<R, FxK<R>::value>(s)
+    GBFFT_FX_SWITCH(T.a.rad[s], CALL)
+#undef CALL
+    __syncthreads();
+  }
+#define CALL(R) T.template last<R, SKIP>(last)
+  GBFFT_FX_SWITCH(T.a.rad[last], CALL)
+#undef CALL
+}
+
+// The rest of a tile with columns that fixed point would shorten: the others,
+// then those in FP64 arithmetic, whose inputs are still there when in == out (the
+// others' outputs lie elsewhere).  Out of line, with passes of its own: one call
+// after the kernel's own passes cost every tile 2 % (registers), and so did a
+// second call inside or the tile handed over by reference (4096 points, 2^24 in
+// all: 234 us so, 237 to 240 otherwise, 232 without any of it).
+template <bool STR>
+__device__ __noinline__ void fx_mixed_tile(const FxArgs& a, unsigned char* smem) {
+  const FxTile<STR, false> T = fx_tile<STR, false>(a, smem);
+  int fixed = 0;
+  for (int c = threadIdx.x; c < T.valid; c += blockDim.x) fixed |= !T.in_fp64(c);
+  if (__syncthreads_or(fixed)) fx_passes<true>(T);
+#pragma unroll 1
+  for (int s = 0; s < a.nrad; ++s) {
+    __syncthreads();
+#define CALL(R) T.template double_pass<R, FxK<R>::value>(s)
+    GBFFT_FX_SWITCH(a.rad[s], CALL)
+#undef CALL
+  }
+}
+
 // 128 registers: one CTA of 512 threads per SM, two of 256, four of 128.
 template <bool STR, bool LIN>
 __global__ void __launch_bounds__(512, 1) fx_kernel(const __grid_constant__ FxArgs a) {
   extern __shared__ __align__(16) unsigned char fx_smem[];
   const FxTile<STR, LIN> T = fx_tile<STR, LIN>(a, fx_smem);
   int* const slot = T.slot;
-  const int last = a.nrad - 1;
   for (int i = threadIdx.x; i < a.nrad * a.C; i += blockDim.x) slot[i] = 0;
   __syncthreads();
-  bool special = false;
-#define CALL(R) special = T.template first<R, FxK<R>::value>()
+  int any = 0;
+#define CALL(R) any = T.template first<R, FxK<R>::value>()
   GBFFT_FX_SWITCH(a.rad[0], CALL)
 #undef CALL
-  if (special) {
-    fx_special_tile<STR, LIN>(T);
+  if (__syncthreads_or(any)) {
+    fx_mixed_tile<STR>(a, fx_smem);
     return;
   }
-  __syncthreads();
-  for (int s = 1; s < last; ++s) {
-#define CALL(R) T.template middle<R, FxK<R>::value>(s)
-    GBFFT_FX_SWITCH(a.rad[s], CALL)
-#undef CALL
-    __syncthreads();
-  }
-#define CALL(R) T.template last<R>(last)
-  GBFFT_FX_SWITCH(a.rad[last], CALL)
-#undef CALL
+  fx_passes<false>(T);
 }
 
 }  // namespace gbfft

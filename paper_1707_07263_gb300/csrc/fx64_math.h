@@ -165,4 +165,18 @@ constexpr int fx_headroom(int r) {
   return r <= 2 ? 2 : r <= 5 ? 3 : r <= 11 ? 4 : 5;
 }
 
+// Which transforms fixed point may take.  An input 2^-k of the largest keeps
+// about 57 - k bits.  Beside a large input of its own sum that is what FP64 keeps
+// of it (the sum rounds it to 53 bits of the larger), but where a whole sum is
+// small the result would lose bits that FP64 holds: real and imaginary parts of
+// different scale, pulses, combs.  So a transform goes to FP64 arithmetic when the
+// real (or the imaginary) inputs of any first-pass butterfly are not all zero
+// and all below 2^-fx_plane_bits of its largest input.  Data of one scale stay:
+// of Gaussian rows of 4096 points, fewer than 1 in 6,000 (radix 2) to 10^18
+// (radix 16) go.
+constexpr int fx_plane_bits(int r) { return 4 + (20 + r - 1) / r; }
+// Row exponents up to this one hold every subnormal number exactly in fixed
+// point (one unit is 2^(E - 1022 - 57)); FP64 products of them would not.
+constexpr int kFxSubnormal = 5;
+
 }  // namespace gbfft

@@ -106,7 +106,7 @@ struct FxArgs {
   const double2* in;
   double2* out;
   const int4* tw;              // Q62 twiddles of every pass, pass s at tw_off[s]: (r - 1) Ns + k
-  const int4* wn;              // W_N^m, m < N (tiles with an infinity or a NaN)
+  const double2* wn;           // W_N^m, m < N (transforms in FP64 arithmetic)
   int N, C;
   int csh, pitch, in_rows;
   int pad_sh, slot_off;        // one pad entry every 2^pad_sh; byte offset of the exponent slots
