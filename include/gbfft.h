@@ -22,6 +22,13 @@
  * fft_exec* never allocates, never synchronises the stream and is safe to
  * capture into a CUDA graph.
  *
+ * Streams and threads: one plan may be executed on several streams and by
+ * several host threads.  Executions that share a workspace (multi-pass plans)
+ * or work counters (uneven batches) run one after another: one on another
+ * stream waits on the device for the last.  A captured execution takes part in
+ * this only as it is captured: order a graph's replays against each other and
+ * against other executions of the plan yourself.
+ *
  * Errors: calls return 0 (FFT_OK) or a negative FFT_ERR_* code; plan
  * constructors return NULL on error.  The code of the last failing call on
  * the calling host thread is kept in fft_last_error().  Argument errors are

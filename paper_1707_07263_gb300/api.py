@@ -175,7 +175,9 @@ _cache_lock = threading.Lock()
 
 
 def get_plan(kind: str, shape, batch: int, prec="fp32", device=None, lengths=None, tuned: bool = False) -> Plan:
-    """Cached plan (twiddle tables are built once per shape/precision/device).
+    """Cached plan (twiddle tables are built once per shape/precision/device),
+    for every stream and thread: the library orders the calls that share its
+    workspace.
     tuned=True builds 1-D and uneven-batch plans from the autotuner's cached
     configuration (tuning the shape first if it has never been tuned on this
     GPU model)."""

@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "../../include/gbfft.h"
 #include "fx64_math.h"
 #include "mixr_plan.h"
@@ -191,6 +193,16 @@ cudaError_t launch_r2c_split64(const double2* z, double2* x, long long M, long l
 cudaError_t launch_c2r_split64(const double2* x, double2* z, long long M, long long batch, const double2* lo,
                                const double2* hi, int s, double end_mul, cudaStream_t st);
 
+// What orders the executions of a plan that share its workspace and counters:
+// the lock keeps one execution's launches together, the event marks the end of
+// the last one, which an execution on another stream waits for on the device.
+struct PlanOrder {
+  std::mutex mu;
+  cudaEvent_t done = nullptr;
+  cudaStream_t last = nullptr;
+  bool ran = false;
+};
+
 }  // namespace gbfft
 
 struct fft_plan {
@@ -262,6 +274,7 @@ struct fft_plan {
   size_t ws_bytes;
   void* ws;
   int ws_owned;
+  gbfft::PlanOrder* order;   // plans whose executions write a workspace or counters (NULL for others)
 
   int* d_status;  // device status word (bounded waits)
 

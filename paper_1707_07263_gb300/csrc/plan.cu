@@ -180,6 +180,8 @@ static fft_plan* new_plan() {
 static void free_plan(fft_plan* p) {
   if (!p) return;
   if (p->inner) free_plan(p->inner);
+  if (p->order && p->order->done) cudaEventDestroy(p->order->done);
+  delete p->order;
   if (p->d_rtw) cudaFree(p->d_rtw);
   if (p->many) many_plan_free(p);
   if (p->fused) fused_plan_free(p);
@@ -1251,6 +1253,14 @@ static std::unordered_set<const fft_plan*>& live_plans() {
 static fft_plan* publish(fft_plan* p) {
   if (!p) return nullptr;
   try {
+    if (p->ws_bytes || p->kind == KIND_MANY) {
+      p->order = new PlanOrder;
+      if (cudaEventCreateWithFlags(&p->order->done, cudaEventDisableTiming) != cudaSuccess) {
+        free_plan(p);
+        set_err(FFT_ERR_CUDA);
+        return nullptr;
+      }
+    }
     std::lock_guard<std::mutex> g(live_mutex());
     live_plans().insert(p);
   } catch (...) {
@@ -1269,6 +1279,31 @@ static bool retire(const fft_plan* p) {
   if (!p) return false;
   std::lock_guard<std::mutex> g(live_mutex());
   return live_plans().erase(p) != 0;
+}
+
+// Runs one execution's launches (call) on stream s after the plan's earlier
+// ones.  An execution on another stream waits on the device for the last one:
+// both write the same workspace.  Under capture the launches go into the graph
+// as they are (an event of another stream would end the capture).
+template <typename Call>
+static int run_ordered(fft_plan* p, cudaStream_t s, const Call& call) {
+  PlanOrder* o = p->order;
+  if (!o) return call();
+  std::lock_guard<std::mutex> g(o->mu);
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    st = cudaStreamCaptureStatusActive;   // the legacy stream while another one captures
+  }
+  if (st != cudaStreamCaptureStatusNone) return call();
+  // (the per-thread default stream has one handle for many streams)
+  if (o->ran && (s != o->last || s == cudaStreamPerThread) && cudaStreamWaitEvent(s, o->done, 0) != cudaSuccess)
+    return FFT_ERR_CUDA;
+  const int rc = call();
+  if (cudaEventRecord(o->done, s) != cudaSuccess) return rc ? rc : FFT_ERR_CUDA;
+  o->last = s;
+  o->ran = true;
+  return rc;
 }
 
 extern "C" {
@@ -1647,12 +1682,13 @@ fft_plan* fft_plan_create_many_config(const int64_t* lengths, int64_t count, int
 
 int fft_exec(fft_plan* plan, const void* in, void* out, void* stream) {
   if (!is_live(plan)) return set_err(FFT_ERR_INVALID_ARG);
-  return set_err(exec_plan(plan, in, out, plan->dir, (cudaStream_t)stream));
+  return fft_exec_dir(plan, in, out, plan->dir, stream);
 }
 
 int fft_exec_dir(fft_plan* plan, const void* in, void* out, int dir, void* stream) {
   if (!is_live(plan)) return set_err(FFT_ERR_INVALID_ARG);
-  return set_err(exec_plan(plan, in, out, dir, (cudaStream_t)stream));
+  return set_err(run_ordered(plan, (cudaStream_t)stream,
+                             [&] { return exec_plan(plan, in, out, dir, (cudaStream_t)stream); }));
 }
 
 int fft_exec_filter_dir(fft_plan* plan, const void* in, void* out, const void* filt, int dir, void* stream) {
@@ -1662,8 +1698,10 @@ int fft_exec_filter_dir(fft_plan* plan, const void* in, void* out, const void* f
   // every launch below reports its own error; one left pending by an earlier,
   // unrelated call must not be taken for this call's
   cudaGetLastError();
-  return set_err(exec_filter_plan(plan, (const float2*)in, (float2*)out, (const float2*)filt,
-                                  dir == FFT_ADJOINT ? 1 : 0, (cudaStream_t)stream));
+  return set_err(run_ordered(plan, (cudaStream_t)stream, [&] {
+    return exec_filter_plan(plan, (const float2*)in, (float2*)out, (const float2*)filt, dir == FFT_ADJOINT ? 1 : 0,
+                            (cudaStream_t)stream);
+  }));
 }
 
 int fft_exec_filter(fft_plan* plan, const void* in, void* out, const void* filt, void* stream) {
