@@ -53,6 +53,14 @@ def _direct(x: torch.Tensor) -> bool:
             and torch._C._get_tracing_state() is None and not torch.compiler.is_compiling())
 
 
+def _plain(x: torch.Tensor) -> torch.Tensor:
+    """x as its memory holds it: contiguous, without the lazy conjugation or
+    negation of a view (x.conj(), x.conj().imag), which a kernel does not see."""
+    if x.is_conj() or x.is_neg():
+        x = x.resolve_conj().resolve_neg()
+    return x.contiguous()
+
+
 class Plan:
     """Owns one library plan and (for four-step plans) its torch-allocated
     workspace.  ``kind`` is "1d", "2d", "many" or "r2c" (real data)."""
@@ -92,6 +100,7 @@ class Plan:
                 raise L.GbfftError(self.lib.fft_last_error(), f"plan {kind} {shape} batch={batch} prec={prec}")
             self.handle = ctypes.c_void_p(h)
             self.points = self.numel()
+            self.dtype = torch.complex128 if self.prec == L.FFT_PREC_FP64 else torch.complex64
             self.ws_bytes = int(self.lib.fft_plan_workspace_bytes(self.handle))
             self.workspace = None
             if self.ws_bytes:
@@ -135,17 +144,18 @@ class Plan:
                  stream=None) -> torch.Tensor:
         if self.kind == "r2c":
             raise TypeError("real plans run through rfft / irfft")
-        want = torch.complex128 if self.prec == L.FFT_PREC_FP64 else torch.complex64
+        want = self.dtype
         if x.dtype != want or not x.is_cuda or x.device != self.device:
             raise TypeError(f"expected a {want} tensor on {self.device}")
         if x.numel() != self.points:
             raise ValueError(f"expected {self.points} elements, got {x.numel()}")
-        x = x.contiguous()
+        x = _plain(x)
         if out is None:
             out = torch.empty_like(x)
         elif (out.dtype != want or out.device != self.device or out.numel() != x.numel()
-              or not out.is_contiguous()):
-            raise ValueError("out must be a contiguous tensor of the input's dtype, device and size")
+              or not out.is_contiguous() or out.is_conj() or out.is_neg()):
+            raise ValueError("out must be a contiguous tensor of the input's dtype, device and size "
+                             "(not a conjugated view)")
         self.exec_ptr(x.data_ptr(), out.data_ptr(), dir, stream)
         return out
 
@@ -232,7 +242,15 @@ def _plan_2d(x, prec):
 
 
 def _run(plan, x, dir):
-    return torch.empty_like(x) if plan is None else plan(x, dir=dir)
+    """plan on x, for which it was looked up (size and device are its own)."""
+    if plan is None:
+        return torch.empty_like(x)
+    if x.dtype != plan.dtype:
+        raise TypeError(f"expected a {plan.dtype} tensor on {plan.device}")
+    x = _plain(x)
+    out = torch.empty_like(x)
+    plan.exec_ptr(x.data_ptr(), out.data_ptr(), dir)
+    return out
 
 
 class _FFT1d(torch.autograd.Function):
@@ -246,7 +264,7 @@ class _FFT1d(torch.autograd.Function):
     def backward(ctx, g):
         if ctx.plan is None:
             return torch.zeros_like(g), None, None
-        return ctx.plan(g.contiguous(), dir=ctx.dir ^ ADJOINT), None, None
+        return ctx.plan(g, dir=ctx.dir ^ ADJOINT), None, None
 
 
 class _FFT2d(torch.autograd.Function):
@@ -260,7 +278,7 @@ class _FFT2d(torch.autograd.Function):
     def backward(ctx, g):
         if ctx.plan is None:
             return torch.zeros_like(g), None, None
-        return ctx.plan(g.contiguous(), dir=ctx.dir ^ ADJOINT), None, None
+        return ctx.plan(g, dir=ctx.dir ^ ADJOINT), None, None
 
 
 class _FFTMany(torch.autograd.Function):
@@ -273,7 +291,7 @@ class _FFTMany(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g):
-        return ctx.plan(g.contiguous(), dir=ctx.dir ^ ADJOINT), None, None, None, None
+        return ctx.plan(g, dir=ctx.dir ^ ADJOINT), None, None, None, None
 
 
 def _prec_for(x: torch.Tensor, prec):
@@ -364,7 +382,7 @@ class _RangeCompress(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g):
         (H,) = ctx.saved_tensors
-        return _run_filter(g.contiguous(), H, ADJOINT), None
+        return _run_filter(_plain(g), H, ADJOINT), None
 
 
 def range_compress(x: torch.Tensor, H: torch.Tensor) -> torch.Tensor:
@@ -378,9 +396,10 @@ def range_compress(x: torch.Tensor, H: torch.Tensor) -> torch.Tensor:
         raise TypeError("H must be a complex64 CUDA tensor of shape (n,)")
     if H.device != x.device:
         raise ValueError("x and H must be on the same device")
+    x, H = _plain(x), _plain(H.detach())
     if _direct(x):
-        return _run_filter(x.contiguous(), H.detach().contiguous())
-    return _RangeCompress.apply(x.contiguous(), H.detach().contiguous())
+        return _run_filter(x, H)
+    return _RangeCompress.apply(x, H)
 
 
 def _run_real(x: torch.Tensor, n: int, dir: int) -> torch.Tensor:
@@ -416,7 +435,7 @@ class _RFFT(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g):
-        return _run_real(g.contiguous(), ctx.n, ADJOINT)
+        return _run_real(_plain(g), ctx.n, ADJOINT)
 
 
 class _IRFFT(torch.autograd.Function):
@@ -432,7 +451,7 @@ class _IRFFT(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g):
-        return _run_real(g.contiguous(), ctx.n, INVERSE | ADJOINT), None
+        return _run_real(_plain(g), ctx.n, INVERSE | ADJOINT), None
 
 
 def rfft(x: torch.Tensor) -> torch.Tensor:
@@ -442,9 +461,10 @@ def rfft(x: torch.Tensor) -> torch.Tensor:
     a 7-smooth FP64 length) -> complex128.  Differentiable."""
     if not isinstance(x, torch.Tensor) or x.dtype not in (torch.float32, torch.float64) or not x.is_cuda:
         raise TypeError("expected a float32 or float64 CUDA tensor")
+    x = _plain(x)
     if _direct(x):
-        return _run_real(x.contiguous(), x.shape[-1], FORWARD)
-    return _RFFT.apply(x.contiguous())
+        return _run_real(x, x.shape[-1], FORWARD)
+    return _RFFT.apply(x)
 
 
 def irfft(X: torch.Tensor, n: int | None = None) -> torch.Tensor:
@@ -457,9 +477,10 @@ def irfft(X: torch.Tensor, n: int | None = None) -> torch.Tensor:
         n = 2 * (X.shape[-1] - 1)
     if X.shape[-1] != n // 2 + 1:
         raise ValueError(f"irfft: {X.shape[-1]} values for length {n}")
+    X = _plain(X)
     if _direct(X):
-        return _run_real(X.contiguous(), int(n), INVERSE)
-    return _IRFFT.apply(X.contiguous(), int(n))
+        return _run_real(X, int(n), INVERSE)
+    return _IRFFT.apply(X, int(n))
 
 
 class HostPipeline:
@@ -511,7 +532,10 @@ class HostPipeline:
         self.last_mode = None
 
     def usable(self, t: torch.Tensor) -> bool:
-        """True if the library's kernels can address t's storage directly."""
+        """True if the library's kernels can address t's storage directly (a
+        conjugated view's storage does not hold its values)."""
+        if t.is_conj() or t.is_neg():
+            return False
         with torch.cuda.device(self.device):
             rc = int(self.lib.fft_pointer_usable(ctypes.c_void_p(t.data_ptr()), t.numel() * t.element_size()))
         if rc < 0:
@@ -542,6 +566,8 @@ class HostPipeline:
             raise TypeError("expected complex64 tensors")
         if x_host.numel() != self.batch * self.n or out_host.numel() != self.batch * self.n:
             raise ValueError("expected batch*n elements")
+        if out_host.is_conj() or out_host.is_neg():
+            raise ValueError("out_host must not be a conjugated view")
         xf, of = x_host.reshape(-1), out_host.reshape(-1)
         cur = torch.cuda.current_stream(self.device)
         direct = self.full_plan is not None and self.usable(xf) and self.usable(of)
@@ -617,6 +643,6 @@ def fft_host(x_host: torch.Tensor, out_host: torch.Tensor | None = None, inverse
     if out_host is None:
         out_host = torch.empty(x_host.shape, dtype=x_host.dtype, pin_memory=torch.cuda.is_available())
     pipe = HostPipeline(n, batch, INVERSE if inverse else FORWARD, chunk=chunk, direct=direct)
-    pipe(x_host.contiguous(), out_host)
+    pipe(_plain(x_host), out_host)
     torch.cuda.synchronize(pipe.device)
     return out_host
