@@ -149,13 +149,21 @@ class Plan:
             raise TypeError(f"expected a {want} tensor on {self.device}")
         if x.numel() != self.points:
             raise ValueError(f"expected {self.points} elements, got {x.numel()}")
-        x = _plain(x)
+        src, x = x, _plain(x)
+        own = [x] if x is not src else []   # tensors made here, on the current stream
         if out is None:
             out = torch.empty_like(x)
+            own.append(out)
         elif (out.dtype != want or out.device != self.device or out.numel() != x.numel()
               or not out.is_contiguous() or out.is_conj() or out.is_neg()):
             raise ValueError("out must be a contiguous tensor of the input's dtype, device and size "
                              "(not a conjugated view)")
+        if own and stream is not None and isinstance(stream, torch.cuda.Stream):
+            current = torch.cuda.current_stream(self.device)
+            if stream != current:
+                stream.wait_stream(current)
+                for t in own:
+                    t.record_stream(stream)
         self.exec_ptr(x.data_ptr(), out.data_ptr(), dir, stream)
         return out
 

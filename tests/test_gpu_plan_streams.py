@@ -105,3 +105,19 @@ def test_captured_after_use_on_another_stream():
     g.replay()
     assert torch.equal(y, ref)
     assert torch.equal(gb.fft(x), ref)
+
+
+def test_explicit_stream_waits_for_what_the_call_makes():
+    """A copy of a strided input and a fresh output are made on the current stream,
+    which is still busy: the other stream's transform comes after them."""
+    p = gb.Plan("1d", (4096,), 64)
+    base = cx(4096, 64)
+    x = base.t()
+    ref = p(x)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        torch.cuda._sleep(20_000_000)
+        y = p(x, stream=s)
+        s.synchronize()
+        assert torch.equal(y, ref)
