@@ -28,10 +28,10 @@ unsigned recip(unsigned d) { return d == 1 ? 0u : (unsigned)((0x100000000ULL + d
 
 }  // namespace
 
-// Entries of the twiddle bases of every pass after the first.
+// Entries of the twiddle tables of every pass after the first.
 size_t mixr_table_entries(const MixrArgs& a) {
   size_t n = 0;
-  for (int s = 1; s < a.nrad; ++s) n += (size_t)log2_up(a.rad[s]) * a.ns[s];
+  for (int s = 1; s < a.nrad; ++s) n += (size_t)(a.rad[s] - 1) * a.ns[s];
   return n;
 }
 
@@ -65,7 +65,7 @@ int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, co
     a.ns[s] = ns;
     a.ns_m[s] = recip(ns);
     a.tw_off[s] = off;
-    if (s > 0) off += (unsigned)log2_up(rad[s]) * ns;
+    if (s > 0) off += (unsigned)(rad[s] - 1) * ns;
     ns *= (unsigned)rad[s];
   }
   a.ncols = ncols;

@@ -16,13 +16,18 @@
 //     writes, so a tile costs 8 bytes a point and several CTAs share an SM;
 //   * the first pass reads global memory and needs no twiddle, the last writes
 //     global memory; each role is its own code, only the radix is switched on;
-//   * the twiddle basis w^(2^e) of every pass is a dense table of Ns columns
-//     (coalesced: lanes hold consecutive k), the other powers are products.
+//   * every twiddle of a pass is an entry of a dense table of Ns columns
+//     (coalesced: lanes hold consecutive k), right to half a unit.  Products of
+//     up to four entries of a basis w^(2^e) are as many instructions but rounded
+//     as often: the largest errors of the transform (9000 points: 1.41e-7 by
+//     products, 1.34e-7 so, 1.37e-7 with the small radices before; 162 to 200000:
+//     2 to 9 % less).  Table against products: 1.2 % more time on average, 0 at
+//     9000 and 15000, 5 at 1000, 6 at most (tiles that leave little L1).
 // Measured on GB300 per 2^25 points, against one pass per prime factor or
 // radix-16 block with two buffers (216 instructions a point and one CTA per SM
-// at N = 9000): 100 173 -> 90 us, 1080 246 -> 113, 7000 340 -> 142, 9000 393 ->
-// 145, 14336 362 -> 206; two passes: 15000 338 -> 206, 10^6 427 -> 302; images
-// of 1000^2 342 -> 253.  (One read and one write of 2^25 points take 79 us.)
+// at N = 9000): 100 173 -> 91 us, 1080 246 -> 114, 7000 340 -> 146, 9000 393 ->
+// 145, 14336 362 -> 206; two passes: 15000 338 -> 207 (1117 of them: 175 -> 112),
+// 10^6 427 -> 280; images of 1000^2 342 -> 258.  (One read and one write of 2^25 points take 79 us.)
 // STR = false: contiguous transforms, element n of transform c at c N + n, in
 // memory and in the tile.  STR = true: C = 2^csh columns, element n of column c
 // at c cs + n ns in memory and n pitch + c in the tile, lanes along columns;
@@ -44,20 +49,13 @@ struct MixrK {
   static constexpr int value = KP / R > 0 ? KP / R : 1;
 };
 
-// v[r] *= w^r with the basis w^(2^e) at tw[e * Ns + k]
+// v[r] *= w^r, w^r at tw[(r - 1) Ns + k]
 template <int R>
 __device__ __forceinline__ void mixr_twiddles(float2* v, const float2* tw, int Ns, int k) {
   float2 w[R];
-  const float2* t = tw + k;
-  ct_for<0, 5>([&](auto ec) __attribute__((always_inline)) {
-    constexpr int e = decltype(ec)::value;
-    if constexpr ((1 << e) < R) w[1 << e] = __ldg(t + e * Ns);
-  });
-  ct_for<3, R>([&](auto rc) __attribute__((always_inline)) {
-    constexpr int r = decltype(rc)::value;
-    constexpr int h = ct_hp2(r);
-    if constexpr (h != r) w[r] = cmul(w[h], w[r - h]);
-  });
+  const float2* t = tw + k;   // (one index (r - 1) Ns + k instead: 4 % slower at 9000)
+#pragma unroll
+  for (int r = 1; r < R; ++r) w[r] = __ldg(t + (r - 1) * Ns);
 #pragma unroll
   for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r]);
 }

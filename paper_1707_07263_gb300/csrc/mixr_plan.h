@@ -60,7 +60,8 @@ inline int log2_up(int r) {
   while ((1 << e) < r) ++e;
   return e;
 }
-// twiddles of a pass: basis loads, products to build the other powers, R - 1 products
+// twiddles of a pass: loads and products of a basis w^(2^e), as they were when the
+// weights below were fitted
 inline float twiddle_cost(int r) {
   const int e = log2_up(r);
   return (2.f * e + 4.f * (r - 1 - e) + 4.f * (r - 1)) / r;
@@ -68,8 +69,10 @@ inline float twiddle_cost(int r) {
 
 // The passes' arithmetic, index work and exchanges.  The weights (and those of
 // tile_cost) are a fit to 9,000 measured (schedule, columns, threads) of 41
-// lengths from 30 to 12288 on GB300: the pick is 0.7 % (at most 5 %) slower
-// than the fastest measured.
+// lengths from 30 to 12288 on GB300: the pick was 0.7 % (at most 5 %) slower than
+// the fastest measured.  With every twiddle from a table it is 1.8 % (at most 11 %)
+// slower than the fastest of 6,605 measured at 44 lengths; weights fitted to those
+// pick better there (0.7 %) but up to 30 % slower at lengths between, so these stay.
 inline float pass_cost_f32(int r, bool first, bool last, bool pad) {
   float per = dft_cost(r) + 10.8f / (float)r + (pad ? 1.6f : 0.f);
   if (!first) per += 1.48f * twiddle_cost(r) + (r >= 15 ? 4.5f : 0.f) + (r >= 20 ? 4.f : 0.f);

@@ -72,20 +72,18 @@ cudaError_t launch_gen_twiddles_step(void* tab, bool fp64, long long N, long lon
   return cudaGetLastError();
 }
 
-// Twiddle basis of one pass of the FP32 mixed-radix tile kernel (mixr.cuh):
-// tab[e * Ns + k] = W_{Ns R}^{2^e k}, k < Ns, every e with 2^e < R.
+// Twiddles of one pass of the FP32 mixed-radix tile kernel (mixr.cuh):
+// tab[(r - 1) Ns + k] = W_{Ns R}^{r k}, 1 <= r < R, k < Ns.
 __global__ void gen_mixr_twiddles(float2* tab, int R, int Ns, int count) {
   const long long M = (long long)Ns * R;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    const int e = i / Ns, k = i - e * Ns;
-    tab[i] = w_entry((long long)k << e, M);
+    const int r = i / Ns + 1, k = i - (r - 1) * Ns;
+    tab[i] = w_entry((long long)r * k, M);
   }
 }
 
 cudaError_t launch_gen_mixr_twiddles(float2* tab, int R, int Ns, cudaStream_t s) {
-  int rows = 0;
-  while ((1 << rows) < R) ++rows;
-  const int count = rows * Ns;
+  const int count = (R - 1) * Ns;
   gen_mixr_twiddles<<<(count + 255) / 256, 256, 0, s>>>(tab, R, Ns, count);
   return cudaGetLastError();
 }
