@@ -62,7 +62,7 @@ struct MixedArgs {
 struct MixrArgs {
   const float2* in;
   float2* out;
-  const float2* tw;            // twiddles of every pass, pass s at tw_off[s]: (r - 1) Ns + k
+  const float2* tw;            // twiddles of every pass, pass s at tw_off[s] (mixr_twiddles)
   int N, C;                    // length; columns per CTA
   int csh, pitch, in_rows;     // strided tiles: C == 2^csh, tile row pitch, input columns are contiguous rows
   int nrad;

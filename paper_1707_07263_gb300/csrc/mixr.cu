@@ -28,10 +28,10 @@ unsigned recip(unsigned d) { return d == 1 ? 0u : (unsigned)((0x100000000ULL + d
 
 }  // namespace
 
-// Entries of the twiddle tables of every pass after the first.
+// Entries of the twiddle tables of every pass after the first (16-byte aligned).
 size_t mixr_table_entries(const MixrArgs& a) {
   size_t n = 0;
-  for (int s = 1; s < a.nrad; ++s) n += (size_t)(a.rad[s] - 1) * a.ns[s];
+  for (int s = 1; s < a.nrad; ++s) n = ((n + 1) & ~(size_t)1) + (size_t)(a.rad[s] - 1) * a.ns[s];
   return n;
 }
 
@@ -64,6 +64,7 @@ int mixr_init(MixrLaunch& L, long long N, long long ncols, long long batches, co
     a.nb_m[s] = recip(a.nb[s]);
     a.ns[s] = ns;
     a.ns_m[s] = recip(ns);
+    off = (off + 1) & ~1u;   // 16-byte pairs
     a.tw_off[s] = off;
     if (s > 0) off += (unsigned)(rad[s] - 1) * ns;
     ns *= (unsigned)rad[s];

@@ -20,14 +20,15 @@
 //     (coalesced: lanes hold consecutive k), right to half a unit.  Products of
 //     up to four entries of a basis w^(2^e) are as many instructions but rounded
 //     as often: the largest errors of the transform (9000 points: 1.41e-7 by
-//     products, 1.34e-7 so, 1.37e-7 with the small radices before; 162 to 200000:
-//     2 to 9 % less).  Table against products: 1.2 % more time on average, 0 at
-//     9000 and 15000, 5 at 1000, 6 at most (tiles that leave little L1).
+//     products, 1.34e-7 so, 1.37e-7 with the small radices before).  Two to a
+//     16-byte load: against products 0.8 % more time on average over 130 lengths
+//     (8-byte loads 1.6 %: 1000 107 us instead of 102, 9000 146 instead of 144), 5
+//     at most (9720, whose tile leaves little L1).
 // Measured on GB300 per 2^25 points, against one pass per prime factor or
 // radix-16 block with two buffers (216 instructions a point and one CTA per SM
-// at N = 9000): 100 173 -> 91 us, 1080 246 -> 114, 7000 340 -> 146, 9000 393 ->
-// 145, 14336 362 -> 206; two passes: 15000 338 -> 207 (1117 of them: 175 -> 112),
-// 10^6 427 -> 280; images of 1000^2 342 -> 258.  (One read and one write of 2^25 points take 79 us.)
+// at N = 9000): 100 173 -> 91 us, 1080 246 -> 114, 7000 340 -> 142, 9000 393 ->
+// 144, 14336 362 -> 205; two passes: 15000 338 -> 207 (1117 of them: 175 -> 112),
+// 10^6 427 -> 282; images of 1000^2 342 -> 252.  (One read and one write of 2^25 points take 79 us.)
 // STR = false: contiguous transforms, element n of transform c at c N + n, in
 // memory and in the tile.  STR = true: C = 2^csh columns, element n of column c
 // at c cs + n ns in memory and n pitch + c in the tile, lanes along columns;
@@ -49,13 +50,19 @@ struct MixrK {
   static constexpr int value = KP / R > 0 ? KP / R : 1;
 };
 
-// v[r] *= w^r, w^r at tw[(r - 1) Ns + k]
+// v[r] *= w^r: pairs (w^{2p+1}, w^{2p+2}) of column k at entry p Ns + k of
+// 16-byte entries, then the last w^r of an even R at one of 8.
 template <int R>
 __device__ __forceinline__ void mixr_twiddles(float2* v, const float2* tw, int Ns, int k) {
-  float2 w[R];
-  const float2* t = tw + k;   // (one index (r - 1) Ns + k instead: 4 % slower at 9000)
+  float2 w[R + 1];
+  const float4* t = (const float4*)tw + k;
 #pragma unroll
-  for (int r = 1; r < R; ++r) w[r] = __ldg(t + (r - 1) * Ns);
+  for (int p = 0; p < (R - 1) / 2; ++p) {
+    const float4 q = __ldg(t + p * Ns);
+    w[2 * p + 1] = make_float2(q.x, q.y);
+    w[2 * p + 2] = make_float2(q.z, q.w);
+  }
+  if constexpr (R % 2 == 0) w[R - 1] = __ldg(tw + (R - 2) * Ns + k);
 #pragma unroll
   for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r]);
 }

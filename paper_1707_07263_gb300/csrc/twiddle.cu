@@ -73,12 +73,14 @@ cudaError_t launch_gen_twiddles_step(void* tab, bool fp64, long long N, long lon
 }
 
 // Twiddles of one pass of the FP32 mixed-radix tile kernel (mixr.cuh):
-// tab[(r - 1) Ns + k] = W_{Ns R}^{r k}, 1 <= r < R, k < Ns.
+// W_{Ns R}^{r k}, 1 <= r < R, k < Ns, in rows of pairs (2p + 1, 2p + 2) and, for
+// an even R, a last row of R - 1 alone.
 __global__ void gen_mixr_twiddles(float2* tab, int R, int Ns, int count) {
   const long long M = (long long)Ns * R;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
     const int r = i / Ns + 1, k = i - (r - 1) * Ns;
-    tab[i] = w_entry((long long)r * k, M);
+    const int last = R % 2 == 0 && r == R - 1;
+    tab[last ? (r - 1) * Ns + k : (((r - 1) >> 1) * Ns + k) * 2 + ((r - 1) & 1)] = w_entry((long long)r * k, M);
   }
 }
 
