@@ -68,7 +68,8 @@ def measured_peaks():
 # register, prefetching and TMA-staged kernels and what they include).  The
 # DRAM traffic recorded in profiles/traffic.json is valid only while these
 # files are unchanged.
-BENCH_KERNEL_SOURCES = ("fft_common.cuh", "fft_radix32.cuh", "tile_fft.cuh", "tile_fft_tma.cuh", "tma_util.cuh", "tile_registry.h",
+BENCH_KERNEL_SOURCES = ("fft_common.cuh", "fft_radix32.cuh", "mixed_ct.cuh", "mixed_common.cuh", "ct_trig.h",
+                        "tile_fft.cuh", "tile_fft_tma.cuh", "tma_util.cuh", "tile_registry.h",
                         "tile_inst_jj.cu", "tile_inst_pf.cu", "tile_inst_tma.cu")
 
 

@@ -75,8 +75,8 @@ enum {
    * about 2^-57 of the row's largest counts only as far as it carries into that
    * unit, which shows where larger inputs cancel exactly.  Transforms whose real
    * or imaginary parts, or some of whose first sums, lie at another scale, and
-   * those with infinities or NaN, run in FP64 arithmetic, at about a fifth of the
-   * speed; one transform's choice does not touch another's.  1-D plans of 7-smooth length
+   * those with infinities or NaN, run in FP64 arithmetic, at a fifth to a seventh
+   * of the speed; one transform's choice does not touch another's.  1-D plans of 7-smooth length
    * n = 2^a 3^b 5^c 7^d (powers of two included): one on-chip pass for
    * 2 <= n <= 7168, two strided passes (four-step, workspace) for
    * 7168 < n <= 7168^2 when n = N1 N2 with N1, N2 <= 7168 (powers of two up

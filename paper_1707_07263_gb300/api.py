@@ -331,7 +331,9 @@ def fft(x: torch.Tensor, prec=None) -> torch.Tensor:
     tensor-core precision): powers of two 2..2^28 and products 2^a 3^b 5^c 7^d
     up to 14336^2 (two passes above 14336).  complex128 runs in FP64: the same
     7-smooth lengths up to 7168^2 (powers of two up to 2^24; two passes above
-    7168)."""
+    7168): in 64-bit integers for rows of one scale (errors below those of FP64
+    sums relative to the row's norm), in FP64 arithmetic for rows that mix scales
+    (see FFT_PREC_FP64 in gbfft.h)."""
     return _apply_1d(x, FORWARD, prec)
 
 

@@ -804,9 +804,9 @@ __global__ void __launch_bounds__(TileCfg<LG, 1, false, false, 0, LGM>::T, LGM =
 }
 
 // Resident CTAs per SM the fused kernel is compiled for: 64 registers per
-// thread at every size (measured on GB300: more registers than the default
-// heuristic picks speed up 2^13 and 2^14; 48 at 256 threads spills and
-// does not help 2^12).
+// thread with radix 16 (measured on GB300: 48 at 256 threads spills and does
+// not help 2^12), 128 with radix 32 (2^13: two CTAs of 256 threads, 2^14: one
+// of 512).
 __host__ __device__ constexpr int rc_min_blocks(int threads, int lgm = 4) {
   const int b = threads <= 256 ? 4 : (threads <= 512 ? 2 : 1);
   return lgm == 5 ? b / 2 : b;   // 128 registers: 32 points a thread
